@@ -87,9 +87,9 @@ typedef enum { GDR_LINK_C128 = 0, GDR_LINK_C64 = 1, GDR_LINK_BF16 = 2 } gdr_link
                                      cycles of the Proj and refinement stages (default: FP32 Givens QR with
                                      one FP64-residual refinement step, the FP64 form when that step's
                                      correction exceeds 1e-4 of the solution) */
-#define GDR_FLAG_NO_TENSOR_CORES 8192u /* MIXED: the projection dot of the Proj and refinement batches over
-                                     the shared kept basis on the CUDA cores (FP32) instead of the tensor
-                                     cores (TF32, tcgen05) */
+#define GDR_FLAG_NO_TENSOR_CORES 8192u /* MIXED: the projection over the shared kept basis of the Proj and
+                                     refinement batches (dot in TF32, update in split TF32) and the restart
+                                     (split TF32) on the CUDA cores (FP32) instead of the tensor cores */
 #define GDR_FLAG_AUTOTUNE   128u  /* before the first cycle, run gdr_autotune for the matvec and Arnoldi
                                      form of each stage whose (precision, columns, m) the operator has
                                      no tuned shape for yet (the tuning time is part of the solve) */
@@ -397,7 +397,10 @@ gdr_status gdr_dense_restart(gdr_ctx *ctx, gdr_prec prec, int m, int k, const do
 /* Basis update (restart, eq. recur1, fused with the multi-shift update):
  * V (n x nv, `prec`) times coefficients C (c128 nv x (nout + nx)):
  * V[:, 0:nout] <- V C[:, 0:nout]  (in place, nout <= nv) and
- * X[:, i] += V C[:, nout + i] for i < nx (X c128 n x nx). */
+ * X[:, i] += V C[:, nout + i] for i < nx (X c128 n x nx).
+ * MIXED with 0 < nout and nout + nx <= 64 runs on the tensor cores (both factors split into
+ * two TF32 parts, FP32 accumulation: FP32 arithmetic's accuracy).  A tensor-core wait that
+ * gave up is reported by the next call that synchronises (GDR_ETIMEOUT). */
 gdr_status gdr_basis_update(gdr_ctx *ctx, gdr_prec prec, long n, int nv, void *V, const double *C, int nout,
                             int nx, double *X);
 

@@ -920,6 +920,7 @@ gdr_status gdr_basis_update(gdr_ctx* ctx, gdr_prec prec, long n, int nv, void* V
   if (!ctx) return GDR_EINVAL;
   return guarded(ctx, [&] {
     GDR_REQUIRE(n > 0 && nv >= 1 && nout >= 0 && nout <= nv && nx >= 0, "bad sizes");
+    ctx->tc_proj = true;
     GDR_REQUIRE(V && C && (nx == 0 || X), "null argument");
     if (prec == GDR_PREC_FP64)
       combine<double>(ctx, n, 1, static_cast<c128*>(V), n, 0, nv, reinterpret_cast<const c128*>(C), nv, 0, nout, nx,

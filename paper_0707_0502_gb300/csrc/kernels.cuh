@@ -159,6 +159,12 @@ bool tc_proj_dot(gdr_ctx* ctx, long n, const c64* V, long ldv, int nv, const c64
 // (nothing launched) when it does not apply.
 bool tc_proj_update(gdr_ctx* ctx, long n, const c64* V, long ldv, int nv, const c128* C, long ccs, int rmode, c64* R,
                     long ldr, int ncol, const ColState* st, int* err, double prof_bytes);
+// GMRES-DR restart on the tensor cores (split TF32, as tc_proj_update): for ncol batch columns
+// with their own bases (stride vcs, lengths nvec), V[:, 0:nout] <- V C[:, 0:nout] in place and
+// X[:, i] += V C[:, nout + i] for i < nx (FP64); C has nv rows at stride ldc, ccs per column.
+// False (nothing launched) when its coefficients do not fit in shared memory.
+bool tc_restart(gdr_ctx* ctx, long n, int ncol, c64* V, long ldv, long vcs, int nv, const c128* C, long ldc, long ccs,
+                int nout, int nx, c128* X, long ldx, long xcs, const ColState* st, const int* nvec, int* err);
 
 // conversions / small vector ops (FP64 <-> complex64)
 void cvt_128_to_64(gdr_ctx* ctx, long n, int cols, const c128* in, long ics, c64* out, long ocs);
