@@ -267,33 +267,17 @@ gdr_status gdr_op_apply(gdr_ctx* ctx, const gdr_op* A, gdr_prec prec, int ncol, 
   return guarded(ctx, [&] {
     GDR_REQUIRE(ncol >= 0 && (ncol == 0 || (sigma && X && Y)), "bad gdr_op_apply arguments");
     if (ncol == 0) return;
-    c128* sd = ctx->get<c128>("apply.sigma", (size_t)ncol);
-    GDR_CUDA(cudaMemcpyAsync(sd, sigma, sizeof(c128) * ncol, cudaMemcpyHostToDevice, ctx->stream));
-    auto run = [&](auto tag) {
-      using R = decltype(tag);
-      const cx<R>* x = static_cast<const cx<R>*>(X);
-      cx<R>* y = static_cast<cx<R>*>(Y);
-      if (A->kind != OP_WILSON) {
-        op_apply<R>(ctx, A, ncol, sd, x, A->n, y, A->n, nullptr, 0);
-        return;
-      }
-      // interface (site-major) order <-> the library's pair-major order
-      cx<R>* xl = ctx->get<cx<R>>("apply.x", (size_t)A->n * ncol);
-      cx<R>* yl = ctx->get<cx<R>>("apply.y", (size_t)A->n * ncol);
-      op_order<cx<R>>(ctx, A, ncol, x, A->n, xl, A->n, true);
-      op_apply<R>(ctx, A, ncol, sd, xl, A->n, yl, A->n, nullptr, 0);
-      op_order<cx<R>>(ctx, A, ncol, yl, A->n, y, A->n, false);
-    };
     if (prec == GDR_PREC_FP64)
-      run(double{});
+      op_apply_user<double>(ctx, A, ncol, sigma, static_cast<const c128*>(X), static_cast<c128*>(Y));
     else
-      run(float{});
+      op_apply_user<float>(ctx, A, ncol, sigma, static_cast<const c64*>(X), static_cast<c64*>(Y));
   });
 }
 
 // Staging of right-hand sides and solutions between the interface order (leading
 // dimension n, host or device memory) and the library order (device, leading dimension
-// ld); Wilson vectors are reordered through a scratch buffer of at most ~256 MB.
+// ld); Wilson vectors in host memory are reordered through a scratch buffer of at most ~256 MB,
+// those in device memory directly.
 static int stage_chunk(const gdr_op* A, long ld, int cols) {
   return (int)std::max<long>(1, std::min<long>(cols, (256L << 20) / (ld * (long)sizeof(c128))));
 }
@@ -303,6 +287,10 @@ static void stage_in(gdr_ctx* ctx, const gdr_op* A, int cols, const double* src,
   if (A->kind != OP_WILSON) {
     GDR_CUDA(cudaMemcpy2DAsync(dst, ld * sizeof(c128), src, n * sizeof(c128), n * sizeof(c128), cols, kind,
                                ctx->stream));
+    return;
+  }
+  if (kind == cudaMemcpyDeviceToDevice) {
+    op_order<c128>(ctx, A, cols, reinterpret_cast<const c128*>(src), n, dst, ld, true);
     return;
   }
   const int ch = stage_chunk(A, ld, cols);
@@ -320,6 +308,10 @@ static void stage_out(gdr_ctx* ctx, const gdr_op* A, int cols, const c128* src, 
   if (A->kind != OP_WILSON) {
     GDR_CUDA(cudaMemcpy2DAsync(dst, n * sizeof(c128), src, ld * sizeof(c128), n * sizeof(c128), cols, kind,
                                ctx->stream));
+    return;
+  }
+  if (kind == cudaMemcpyDeviceToDevice) {
+    op_order<c128>(ctx, A, cols, src, ld, reinterpret_cast<c128*>(dst), n, false);
     return;
   }
   const int ch = stage_chunk(A, ld, cols);

@@ -185,13 +185,16 @@ void op_apply_skip(gdr_ctx* ctx, const gdr_op* A, int ncol, const c128* sigma, c
 void op_apply_skip(gdr_ctx* ctx, const gdr_op* A, int ncol, const c128* sigma, const c64* X, long ldx, c64* Y,
                    long ldy, const c64* B, long ldb, const int* run, int run_stride, int cpp = 1,
                    const double* xs = nullptr, int xs_stride = 0);
+// Y[:, c] = (A - sigma_c) X[:, c] for vectors in the C interface's order, shifts on the host
+template <typename R>
+void op_apply_user(gdr_ctx* ctx, const gdr_op* A, int ncol, const double* sigma, const cx<R>* X, cx<R>* Y);
 // launch shape of the operator kernels for ncol columns (FP64 or complex64 vectors): the
 // shape set for this column count, else the one set for the nearest count within a
 // factor 2, else the defaults (Wilson: direction-split while one thread per site cannot
-// fill the GPU; CSR: one thread per row; several columns of one operator in column-inner
-// block order)
+// fill the GPU, column pairs for several complex64 columns; CSR: one thread per row; several
+// columns of one operator in column-inner block order unless its links stay in L2)
 MvShape mv_shape(const gdr_ctx* ctx, const gdr_op* A, bool f64, int ncol);
-MvShape mv_default(const gdr_ctx* ctx, const gdr_op* A, int ncol);
+MvShape mv_default(const gdr_ctx* ctx, const gdr_op* A, bool f64, int ncol);
 // Vector order: the C interface passes Wilson vectors site-major, the library keeps
 // them pair-major (see wilson.cuh).  to_lib: interface -> library order, else back.
 // Other operators: a plain copy (none when in == out).  in and out must differ.

@@ -112,7 +112,7 @@ static void tune_matvec(gdr_ctx* ctx, gdr_op* A, int ncol, gdr_tune_result& out)
   auto run = [&] { op_apply<R>(ctx, A, ncol, nullptr, X, ld, Y, ld, nullptr, 0, cpp); };
 
   A->mv_tuned.erase(key);
-  const MvShape def = mv_default(ctx, A, ncol);
+  const MvShape def = mv_default(ctx, A, F64, ncol);
   MvShape best = def;
   double tbest = 1e30, tdef = -1;
   int count = 0;
