@@ -148,6 +148,7 @@ gdr_status gdr_create(gdr_ctx** out, int device, void* cuda_stream) {
     }
     dense_init(ctx);
     krylov_init(ctx);
+    dcgs2_init(ctx);
     sweep_init(ctx);
     tc_proj_init(ctx);
   });
@@ -769,6 +770,7 @@ gdr_status gdr_arnoldi_cycle(gdr_ctx* ctx, const gdr_op* A, gdr_prec prec, void*
       GDR_CUDA(cudaStreamSynchronize(ctx->stream));
       if (m_eff) *m_eff = out.broke ? out.m_eff : m;
       if (out.nan) throw gdr_error(GDR_ENAN, "NaN/Inf in the Arnoldi recurrence");
+      if (out.err) throw gdr_error((gdr_status)out.err, "a wait in the Arnoldi recurrence gave up");
     };
     if (prec == GDR_PREC_FP64)
       run(double{});

@@ -36,7 +36,7 @@ struct Batch {
   c128* cvec = nullptr;  // m+1 per column
   c128* h1 = nullptr;    // (m+2) per column: GS dots (+ ||w||^2 in slot m+1)
   c128* h2 = nullptr;
-  c128* hd = nullptr;    // DCGS2 dot values per column (2m + 8), see arnoldi_dcgs2
+  c128* hd = nullptr;    // DCGS2 projections of a step per column (2m + 8), see dcgs2.cu
   c128* dc = nullptr;    // DCGS2 update coefficients per column (2m + 8)
   c64* Hf = nullptr;     // DCGS2: FP32 copy of H (same layout), for the small H s correction
   c128* part = nullptr;  // block partials, per column pstride
@@ -104,6 +104,11 @@ void arnoldi_step(gdr_ctx* ctx, const gdr_op* A, const Batch<R>& b, int j, int j
 // and partials of (2m + 8) values per slot.
 template <typename R>
 void arnoldi_dcgs2(gdr_ctx* ctx, const gdr_op* A, const Batch<R>& b, int jstart, int jend);
+template <>
+void arnoldi_dcgs2<float>(gdr_ctx*, const gdr_op*, const Batch<float>&, int, int);
+template <>
+void arnoldi_dcgs2<double>(gdr_ctx*, const gdr_op*, const Batch<double>&, int, int);
+void dcgs2_init(gdr_ctx* ctx);
 // persistent Arnoldi sweep (sweep.cu): steps jstart..jend-1 of every column in one
 // cooperative launch; v_jend is left unnormalised in W2 (scale_into writes it).
 // sweep_fits: short vectors, where the sweep replaces the per-phase launches.
