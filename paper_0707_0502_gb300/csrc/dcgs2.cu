@@ -61,6 +61,56 @@ DEV float warp_sum4(c64 a, c64 w, int lane) {
   return r;
 }
 
+// the same for three FP64 values, six additions instead of fifteen (an FP64 instruction holds
+// its pipe for ~64 cycles a warp).  Lanes 0, 8, 16 hold x, y, z.
+DEV double warp_sum3(double x, double y, double z, int lane) {
+  const bool h16 = lane & 16, h8 = lane & 8;
+  double k0 = h16 ? z : x, k1 = h16 ? 0.0 : y;
+  k0 += __shfl_xor_sync(FULL, h16 ? x : z, 16);
+  k1 += __shfl_xor_sync(FULL, h16 ? y : 0.0, 16);
+  double r = h8 ? k1 : k0;
+  r += __shfl_xor_sync(FULL, h8 ? k0 : k1, 8);
+  r += __shfl_xor_sync(FULL, r, 4);
+  r += __shfl_xor_sync(FULL, r, 2);
+  r += __shfl_xor_sync(FULL, r, 1);
+  return r;
+}
+
+// 1/sqrt(x) for a positive normal x: Newton's iteration y <- y + y/2 (1 - x y^2) from an
+// FP32 starting value (x scaled by a power of four into its range), 2^-22 -> 2^-43 -> FP64
+// rounding: nine dependent FP64 instructions where sqrt and a division take over twenty.
+DEV double rsqrt_newton(double x) {
+  const long long bits = __double_as_longlong(x);
+  const int e = (int)((bits >> 52) & 0x7ff) - 1023, h = e >> 1;  // x = 4^h xs, xs in [1, 4)
+  const double xs = __longlong_as_double(bits - (long long)(2 * h) * (1LL << 52));
+  double y = (double)rsqrtf((float)xs);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const double r = fma(-xs * y, y, 1.0);
+    y = fma(0.5 * y, r, y);
+  }
+  return y * __longlong_as_double((long long)(1023 - h) * (1LL << 52));
+}
+
+// atomicAdd that releases the block's earlier writes (all threads', ordered before by a block
+// barrier) and acquires those of the blocks that came before: no fence per thread
+DEV unsigned ticket(unsigned* p) {
+  unsigned r;
+  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(r) : "l"(p) : "memory");
+  return r;
+}
+
+// sum over the slots q0..q1-1 of part[q * hs + i], by two neighbouring lanes (even, odd slots),
+// valid in both
+DEV c128 slot_sum2(const c128* part, int hs, int i, int q0, int q1, int half) {
+  c128 acc = {0, 0};
+#pragma unroll 8
+  for (int q = q0 + half; q < q1; q += 2) acc += ldcg128(part + (long)q * hs + i);
+  acc.x += __shfl_xor_sync(FULL, acc.x, 1);
+  acc.y += __shfl_xor_sync(FULL, acc.y, 1);
+  return acc;
+}
+
 // Dot pass.  HBM bounds it (V_j read once, u and w once), so what matters is bytes in
 // flight.  Each warp holds its slab of u and w (du <= 8 units per lane) in registers and
 // streams the vectors of its group through it from a ring of its own in shared memory,
@@ -71,7 +121,7 @@ __global__ void __launch_bounds__(NT, 2) dcgs2_dot_kernel(Batch<float> b, int j,
                                                        const c64* __restrict__ W, long wcs, int S, int G, int du,
                                                        int mode) {
   const int c = blockIdx.y;
-  if (!b.st[c].run) return;
+  const int run = b.st[c].run;  // tested once the barriers are set up
   extern __shared__ __align__(128) unsigned char ring_raw[];
   __shared__ c64 accw[NW][2 * GDR_MAX_M + 8];
   __shared__ __align__(8) uint64_t full[NW][NST];
@@ -92,6 +142,7 @@ __global__ void __launch_bounds__(NT, 2) dcgs2_dot_kernel(Batch<float> b, int j,
   if (threadIdx.x == 0) abort_s = 0;
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   for (int v = v0 + lane; v < v1; v += 32) accw[warp][v] = {0, 0};
+  if (!run) return;
   __syncthreads();
   const int SU = 32 * du;  // units per slab
   const long nslab = i0 < i1 ? (nu + SU - 1) / SU : 0, dsl = (long)S * NW;
@@ -197,45 +248,40 @@ __global__ void __launch_bounds__(NT, 2) dcgs2_dot_kernel(Batch<float> b, int j,
 
   // ---- two-level sum over the slots, into shared memory of the last block
   __shared__ bool last_s;
-  __shared__ double red_d[NW];
-  __shared__ c128 red_c[NW];
+  __shared__ double red_s[NW][4];  // |s|^2, Re and Im of s^H z
+  __shared__ double wn_s;
   __shared__ c128 t_s;
   __shared__ int brk_s;
   c128* sval = reinterpret_cast<c128*>(ring_raw);  // the ring has been read
   const int nval = 2 * j + 3, ng = (S + RG - 1) / RG, rg = slot / RG;
   c128* gpart = part + (long)b.nblk * hs;
-  __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
     const unsigned nbg = (unsigned)(min(S, (rg + 1) * RG) - rg * RG) * (unsigned)G;
-    last_s = atomicAdd(&b.gcnt[64 * c + rg], 1u) == nbg - 1;
+    last_s = ticket(&b.gcnt[64 * c + rg]) == nbg - 1;
   }
   __syncthreads();
   if (!last_s) return;
-  __threadfence();
-  {
-    const int s0 = rg * RG, s1 = min(S, s0 + RG);
-    for (int i = threadIdx.x; i < nval; i += NT) {
-      c128 acc = {0, 0};
-#pragma unroll 8
-      for (int q = s0; q < s1; ++q) acc += ldcg128(part + (long)q * hs + i);
-      if (ng == 1) sval[i] = acc;
-      else gpart[(long)rg * hs + i] = acc;
-    }
+  const int half = threadIdx.x & 1;
+  for (int ib = 0; ib < nval; ib += NT / 2) {
+    const int i = ib + (int)(threadIdx.x >> 1), s0 = rg * RG, s1 = i < nval ? min(S, s0 + RG) : s0;
+    const c128 acc = slot_sum2(part, hs, i, s0, s1, half);
+    if (half || i >= nval) continue;
+    if (ng == 1) sval[i] = acc;
+    else gpart[(long)rg * hs + i] = acc;
   }
   if (ng > 1) {
-    __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) last_s = atomicAdd(&b.cnt[4 * c + 1], 1u) == (unsigned)ng - 1;
+    if (threadIdx.x == 0) {
+      b.gcnt[64 * c + rg] = 0;
+      last_s = ticket(&b.cnt[4 * c + 1]) == (unsigned)ng - 1;
+    }
     __syncthreads();
-    if (threadIdx.x == 0) b.gcnt[64 * c + rg] = 0;
     if (!last_s) return;
-    __threadfence();
-    for (int i = threadIdx.x; i < nval; i += NT) {
-      c128 acc = {0, 0};
-#pragma unroll 8
-      for (int g = 0; g < ng; ++g) acc += ldcg128(gpart + (long)g * hs + i);
-      sval[i] = acc;
+    for (int ib = 0; ib < nval; ib += NT / 2) {
+      const int i = ib + (int)(threadIdx.x >> 1);
+      const c128 acc = slot_sum2(gpart, hs, i, 0, i < nval ? ng : 0, half);
+      if (!half && i < nval) sval[i] = acc;
     }
     if (threadIdx.x == 0) b.cnt[4 * c + 1] = 0;
   } else if (threadIdx.x == 0) {
@@ -255,19 +301,12 @@ __global__ void __launch_bounds__(NT, 2) dcgs2_dot_kernel(Batch<float> b, int j,
       if (!first) si = sval[2 * i];
       zi = sval[2 * i + 1];
     }
-    double ssp = norm2(si);
-    c128 szp = cmulc(si, zi);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      ssp += __shfl_xor_sync(FULL, ssp, off);
-      szp.x += __shfl_xor_sync(FULL, szp.x, off);
-      szp.y += __shfl_xor_sync(FULL, szp.y, off);
-    }
-    if (lane == 0) {
-      red_d[warp] = ssp;
-      red_c[warp] = szp;
-    }
+    const c128 szp = cmulc(si, zi);
+    const double r = warp_sum3(norm2(si), szp.x, szp.y, lane);
+    if ((lane & 7) == 0) red_s[warp][lane >> 3] = r;
   }
+  // beside it, on another warp's pipe: ||w||
+  if (threadIdx.x == NT - 32) wn_s = mode != DC_FINAL ? sqrt(sval[2 * j + 2].x) : 0.0;
   __syncthreads();
   ColState& st = b.st[c];
   c128* hv = b.hd + (long)c * hs;
@@ -276,11 +315,15 @@ __global__ void __launch_bounds__(NT, 2) dcgs2_dot_kernel(Batch<float> b, int j,
     double ss = 0;
     c128 sz = {0, 0};
     for (int q = 0; q < nwj; ++q) {
-      ss += red_d[q];
-      sz += red_c[q];
+      ss += red_s[q][0];
+      sz += c128{red_s[q][1], red_s[q][2]};
     }
     const double omega = sval[2 * j].x;
-    const double nuv = first ? 1.0 : sqrt(fmax(omega - ss, 0.0));
+    // nu and 1/nu by the iteration where nu^2 is in its range, else by sqrt and a division
+    const double nu2 = fmax(omega - ss, 0.0);
+    const bool plain = nu2 > 1e-290 && nu2 < 1e290;
+    double inu = first ? 1.0 : plain ? rsqrt_newton(nu2) : 0.0;
+    const double nuv = first ? 1.0 : plain ? nu2 * inu : sqrt(nu2);
     int brk = 0;
     if (!first) {
       if (!isfinite(nuv) || !isfinite(omega)) {
@@ -297,7 +340,7 @@ __global__ void __launch_bounds__(NT, 2) dcgs2_dot_kernel(Batch<float> b, int j,
       }
     }
     if (!brk) {
-      const double inu = 1.0 / nuv;
+      if (!first && !plain) inu = 1.0 / nuv;
       st.inv_norm = inu;
       st.j = j;
       hv[2 * j] = {nuv, 0.0};
@@ -307,9 +350,8 @@ __global__ void __launch_bounds__(NT, 2) dcgs2_dot_kernel(Batch<float> b, int j,
         df[2 * (m + 1)] = to64(tn);
         hv[2 * j + 1] = t;
         t_s = tn;
-        const double ww = sval[2 * j + 2].x;
-        st.wnorm0 = sqrt(ww) * inu;
-        if (!isfinite(ww)) {
+        st.wnorm0 = wn_s * inu;
+        if (!isfinite(wn_s)) {
           st.nan = 1;
           st.broke = 1;
           st.run = 0;
