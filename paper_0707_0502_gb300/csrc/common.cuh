@@ -39,6 +39,43 @@ template <typename R> HD cx<R> conj(cx<R> a) { return {a.x, -a.y}; }
 template <typename R> HD R norm2(cx<R> a) { return a.x * a.x + a.y * a.y; }
 // conj(a) * b
 template <typename R> HD cx<R> cmulc(cx<R> a, cx<R> b) { return {a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x}; }
+// acc + a b, acc - a b, acc + conj(a) b as four FMAs (a product and an addition are six
+// floating-point instructions, and the FP64 pipe bounds most FP64 kernels here)
+template <typename R> HD cx<R> cfma(cx<R> c, cx<R> a, cx<R> b) {
+  return {fma(-a.y, b.y, fma(a.x, b.x, c.x)), fma(a.y, b.x, fma(a.x, b.y, c.y))};
+}
+template <typename R> HD cx<R> cfnma(cx<R> c, cx<R> a, cx<R> b) {
+  return {fma(a.y, b.y, fma(-a.x, b.x, c.x)), fma(-a.y, b.x, fma(-a.x, b.y, c.y))};
+}
+// A long sum of such products in two accumulators, the terms with a.x and those with a.y
+// apart: one rounding per accumulator and term, as with the products formed first (chained
+// FMAs into one accumulator round twice)
+template <typename R>
+struct CSum {
+  cx<R> p = {0, 0}, q = {0, 0};
+  HD void mac(cx<R> a, cx<R> b) {  // += a b
+    p = {fma(a.x, b.x, p.x), fma(a.x, b.y, p.y)};
+    q = {fma(-a.y, b.y, q.x), fma(a.y, b.x, q.y)};
+  }
+  HD void macc(cx<R> a, cx<R> b) {  // += conj(a) b
+    p = {fma(a.x, b.x, p.x), fma(a.x, b.y, p.y)};
+    q = {fma(a.y, b.y, q.x), fma(-a.y, b.x, q.y)};
+  }
+  HD void norm(cx<R> a) {  // += |a|^2
+    p.x = fma(a.x, a.x, p.x);
+    q.x = fma(a.y, a.y, q.x);
+  }
+  HD cx<R> value() const { return {p.x + q.x, p.y + q.y}; }
+};
+// FP32 kernels are bound by memory and registers: one accumulator, the products first
+template <>
+struct CSum<float> {
+  c64 p = {0, 0};
+  HD void mac(c64 a, c64 b) { p += a * b; }
+  HD void macc(c64 a, c64 b) { p += cmulc(a, b); }
+  HD void norm(c64 a) { p.x += norm2(a); }
+  HD c64 value() const { return p; }
+};
 // i * a
 template <typename R> HD cx<R> mul_i(cx<R> a) { return {-a.y, a.x}; }
 HD c128 to128(c64 a) { return {(double)a.x, (double)a.y}; }

@@ -24,6 +24,19 @@ DEV c128 ldcg128(const c128* p) {
   return {v.x, v.y};
 }
 
+// Sum of a complex value over the warp, by halving: the first exchange splits the parts over
+// the half-warps, so each lane adds five times instead of ten.  Valid in every lane.
+template <typename R>
+DEV cx<R> warp_sum(cx<R> a, int lane) {
+  const bool h = lane & 16;
+  R k = h ? a.y : a.x;
+  k += __shfl_xor_sync(FULL, h ? a.x : a.y, 16);
+#pragma unroll
+  for (int off = 8; off > 0; off >>= 1) k += __shfl_xor_sync(FULL, k, off);
+  const R o = __shfl_xor_sync(FULL, k, 16);
+  return h ? cx<R>{o, k} : cx<R>{k, o};
+}
+
 // Reduce NV complex values over the block; threads < nvalid write out[t].
 template <typename R, int NV>
 DEV void block_reduce(cx<R> (&acc)[NV], c128* out, int nvalid) {
@@ -167,49 +180,49 @@ __global__ void __launch_bounds__(NT, 3) gs_dot_kernel(Batch<R> b, int nv, const
     }
     __syncthreads();
     for (int i = i0 + warp; i < i1; i += NT / 32) {
-      cx<R> a = {0, 0};
+      CSum<R> acc;
       if (i < nv) {
         // lazy step: v_{nv-1} is the previous step's unnormalised vector; scale it
         // and store it into V while it is read
         const bool lazy = Wprev && i == nv - 1;
         const cx<R>* vi = lazy ? Wprev + c * wcs : V + (long)i * b.ldv;
-        cx<R> vv[DU][K];
+        constexpr int LB = sizeof(R) == 8 ? 8 : DU;  // units loaded together
 #pragma unroll
-        for (int tt = 0; tt < DU; ++tt) {
-          const long u = u0 + lane + 32 * tt;
-          if (u < nu) {
-            ldu<R>(vi, u, n, vv[tt]);
-          } else {
+        for (int t0 = 0; t0 < DU; t0 += LB) {
+          cx<R> vv[LB][K];
 #pragma unroll
-            for (int kk = 0; kk < K; ++kk) vv[tt][kk] = {0, 0};
+          for (int tt = 0; tt < LB; ++tt) {
+            const long u = u0 + lane + 32 * (t0 + tt);
+            if (u < nu) {
+              ldu<R>(vi, u, n, vv[tt]);
+            } else {
+#pragma unroll
+              for (int kk = 0; kk < K; ++kk) vv[tt][kk] = {0, 0};
+            }
           }
-        }
-        if (lazy) {
-          const R sc = (R)b.st[c].inv_norm;
-          cx<R>* vo = b.V + c * b.vcs + (long)i * b.ldv;
+          if (lazy) {
+            const R sc = (R)b.st[c].inv_norm;
+            cx<R>* vo = b.V + c * b.vcs + (long)i * b.ldv;
 #pragma unroll
-          for (int tt = 0; tt < DU; ++tt) {
+            for (int tt = 0; tt < LB; ++tt) {
 #pragma unroll
-            for (int kk = 0; kk < K; ++kk) vv[tt][kk] = sc * vv[tt][kk];
-            const long u = u0 + lane + 32 * tt;
-            if (u < nu) stu<R>(vo, u, n, vv[tt]);
+              for (int kk = 0; kk < K; ++kk) vv[tt][kk] = sc * vv[tt][kk];
+              const long u = u0 + lane + 32 * (t0 + tt);
+              if (u < nu) stu<R>(vo, u, n, vv[tt]);
+            }
           }
+#pragma unroll
+          for (int tt = 0; tt < LB; ++tt)
+#pragma unroll
+            for (int kk = 0; kk < K; ++kk) acc.macc(vv[tt][kk], wt[(lane + 32 * (t0 + tt)) * K + kk]);
         }
-#pragma unroll
-        for (int tt = 0; tt < DU; ++tt)
-#pragma unroll
-          for (int kk = 0; kk < K; ++kk) a += cmulc(vv[tt][kk], wt[(lane + 32 * tt) * K + kk]);
       } else {  // ||w||^2
 #pragma unroll
         for (int tt = 0; tt < DU; ++tt)
 #pragma unroll
-          for (int kk = 0; kk < K; ++kk) a.x += norm2(wt[(lane + 32 * tt) * K + kk]);
+          for (int kk = 0; kk < K; ++kk) acc.norm(wt[(lane + 32 * tt) * K + kk]);
       }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        a.x += __shfl_xor_sync(FULL, a.x, off);
-        a.y += __shfl_xor_sync(FULL, a.y, off);
-      }
+      const cx<R> a = warp_sum(acc.value(), lane);
       if (lane == 0) accs[i] += up(a);
     }
   }
@@ -259,6 +272,7 @@ __global__ void __launch_bounds__(NT, 2) gs_update_dot_kernel(Batch<R> b, int nv
       cx<R> acc[K];
       if (u < nu) {
         ldu<R>(w, u, n, acc);
+        CSum<R> sum[K];
         for (int g0 = 0; g0 < nv; g0 += JB) {
           cx<R> vv[JB][K];
 #pragma unroll
@@ -269,10 +283,12 @@ __global__ void __launch_bounds__(NT, 2) gs_update_dot_kernel(Batch<R> b, int nv
             if (g0 + qq < nv) {
               const cx<R> hi = hs[g0 + qq];
 #pragma unroll
-              for (int kk = 0; kk < K; ++kk) acc[kk] -= vv[qq][kk] * hi;
+              for (int kk = 0; kk < K; ++kk) sum[kk].mac(vv[qq][kk], hi);
             }
           }
         }
+#pragma unroll
+        for (int kk = 0; kk < K; ++kk) acc[kk] -= sum[kk].value();
         if (grp == 0) stu<R>(wo, u, n, acc);
       } else {
 #pragma unroll
@@ -284,7 +300,7 @@ __global__ void __launch_bounds__(NT, 2) gs_update_dot_kernel(Batch<R> b, int nv
     __syncthreads();
     for (int i = i0 + warp; i < i1; i += NT / 32) {
       const cx<R>* vi = V + (long)i * b.ldv;
-      cx<R> a = {0, 0};
+      CSum<R> acc;
       // the tile in two halves (DU/2 loads in flight per lane; the tile is in L1/L2)
 #pragma unroll
       for (int t0 = 0; t0 < DU; t0 += DU / 2) {
@@ -302,13 +318,9 @@ __global__ void __launch_bounds__(NT, 2) gs_update_dot_kernel(Batch<R> b, int nv
 #pragma unroll
         for (int tt = 0; tt < DU / 2; ++tt)
 #pragma unroll
-          for (int kk = 0; kk < K; ++kk) a += cmulc(vv[tt][kk], wt[(lane + 32 * (t0 + tt)) * K + kk]);
+          for (int kk = 0; kk < K; ++kk) acc.macc(vv[tt][kk], wt[(lane + 32 * (t0 + tt)) * K + kk]);
       }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        a.x += __shfl_xor_sync(FULL, a.x, off);
-        a.y += __shfl_xor_sync(FULL, a.y, off);
-      }
+      const cx<R> a = warp_sum(acc.value(), lane);
       if (lane == 0) accs[i] += up(a);
     }
   }
@@ -337,6 +349,7 @@ __global__ void __launch_bounds__(NT) gs_update_kernel(Batch<R> b, int nv, cx<R>
   cx<R> nrm[1] = {{0, 0}};
   for (long u = gt; u < nu; u += gs) {
     cx<R> acc[K];
+    CSum<R> sum[K];
     ldu<R>(w, u, n, acc);
     // basis vectors in groups of JB: all loads of a group are in flight together
     for (int i0 = 0; i0 < nv; i0 += JB) {
@@ -350,13 +363,15 @@ __global__ void __launch_bounds__(NT) gs_update_kernel(Batch<R> b, int nv, cx<R>
         if (i0 + q < nv) {
           const cx<R> hi = hs[i0 + q];
 #pragma unroll
-          for (int kk = 0; kk < K; ++kk) acc[kk] -= vv[q][kk] * hi;
+          for (int kk = 0; kk < K; ++kk) sum[kk].mac(vv[q][kk], hi);
         }
       }
     }
+#pragma unroll
+    for (int kk = 0; kk < K; ++kk) acc[kk] -= sum[kk].value();
     stu<R>(w, u, n, acc);
 #pragma unroll
-    for (int kk = 0; kk < K; ++kk) nrm[0].x += norm2(acc[kk]);
+    for (int kk = 0; kk < K; ++kk) nrm[0].x = fma(acc[kk].y, acc[kk].y, fma(acc[kk].x, acc[kk].x, nrm[0].x));
   }
   if (!final_step) return;
   c128* part = b.part + c * b.pstride;
@@ -445,7 +460,7 @@ __global__ void __launch_bounds__(NT) norms2_kernel(long n, const T* __restrict_
   }
   for (; i < n; i += stride) {
     const T v = xc[i];
-    s += (double)v.x * v.x + (double)v.y * v.y;
+    s = fma((double)v.y, (double)v.y, fma((double)v.x, (double)v.x, s));
   }
   c128 d[1] = {{s, 0}};
   block_reduce<double, 1>(d, part + (long)c * gridDim.x + blockIdx.x, 1);
@@ -465,8 +480,9 @@ __global__ void __launch_bounds__(NT) dots128_kernel(long n, const c128* __restr
   const int c = blockIdx.y;
   const c128* uc = u + c * ucs;
   const c128* xc = x + c * xcs;
-  c128 a[1] = {{0, 0}};
-  for (long i = blockIdx.x * (long)NT + threadIdx.x; i < n; i += (long)gridDim.x * NT) a[0] += cmulc(uc[i], xc[i]);
+  CSum<double> sum;
+  for (long i = blockIdx.x * (long)NT + threadIdx.x; i < n; i += (long)gridDim.x * NT) sum.macc(uc[i], xc[i]);
+  c128 a[1] = {sum.value()};
   block_reduce<double, 1>(a, part + (long)c * gridDim.x + blockIdx.x, 1);
   if (!last_block(cnt + 4 * c)) return;
   if (threadIdx.x < 32) {
@@ -550,7 +566,11 @@ __global__ void __launch_bounds__(CT) combine_kernel(long n, cx<R>* V, long ldv,
   for (int o = threadIdx.x / CR; o < ntot; o += CT / CR) {
     cx<R> acc = {0, 0};
     const cx<R>* co = cf + (long)o * nv;
-    for (int i = 0; i < nv; ++i) acc += tile[(long)i * CR + rr] * co[i];
+    if constexpr (sizeof(R) == 8) {
+      for (int i = 0; i < nv; ++i) acc = cfma(acc, tile[(long)i * CR + rr], co[i]);
+    } else {
+      for (int i = 0; i < nv; ++i) acc += tile[(long)i * CR + rr] * co[i];
+    }
     if (o < nout) {
       Vc[(long)o * ldv + row] = acc;
     } else if (o < nout + nx) {
@@ -602,7 +622,7 @@ __global__ void __launch_bounds__(256) combine_rows_kernel(long n, const cx<R>* 
       const cx<R> v = Vc[(long)i * ldv + row];
 #pragma unroll
       for (int o = 0; o < NO; ++o)
-        if (o < ntot) acc[o] += v * cf[o * nv + i];
+        if (o < ntot) acc[o] = sizeof(R) == 8 ? cfma(acc[o], v, cf[o * nv + i]) : acc[o] + v * cf[o * nv + i];
     }
 #pragma unroll
     for (int o = 0; o < NO; ++o) {
@@ -673,7 +693,7 @@ __global__ void __launch_bounds__(CT) combine_shared_kernel(long n, const cx<R>*
       for (int i = 0; i < nv; ++i) {
         const cx<R> t = tile[(long)i * CR + rr];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q] += t * co[q][i];
+        for (int q = 0; q < 4; ++q) acc[q] = sizeof(R) == 8 ? cfma(acc[q], t, co[q][i]) : acc[q] + t * co[q][i];
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -757,7 +777,10 @@ __global__ void __launch_bounds__(DS_W * 32) gs_dot_shared_kernel(long n, const 
     for (int i = 0; i < NVM; ++i) {
       if (i >= nv) break;
 #pragma unroll
-      for (int q = 0; q < DS_EPL; ++q) acc[i] += cmulc(vt[i * DS_TR + lane + 32 * q], rv[q]);
+      for (int q = 0; q < DS_EPL; ++q) {
+        const cx<R> v = vt[i * DS_TR + lane + 32 * q];
+        acc[i] = sizeof(R) == 8 ? cfma(acc[i], conj(v), rv[q]) : acc[i] + cmulc(v, rv[q]);
+      }
     }
     if (++cnt == DS_FL) {
       flush();
@@ -803,7 +826,7 @@ __global__ void axpy_cols_kernel(long n, const c128* a, const c128* S, long ssc,
   const int c = blockIdx.y;
   const c128 ac = a[c];
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-    X[c * xcs + i] += ac * S[c * ssc + i];
+    X[c * xcs + i] = cfma(X[c * xcs + i], ac, S[c * ssc + i]);
 }
 __global__ void scal_cols_kernel(long n, const c128* a, c128* X, long xcs) {
   const int c = blockIdx.y;

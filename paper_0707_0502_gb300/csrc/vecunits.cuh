@@ -40,7 +40,8 @@ template <> DEV void stu<double>(c128* p, long u, long, const c128 (&o)[1]) {
 }
 template <typename R> HD long nunits(long n) { return (n + U<R>::K - 1) / U<R>::K; }
 
-// units per lane of a dot tile (a tile of w is DU * 32 units)
-template <typename R> struct DotTile { static constexpr int DU = (U<R>::K == 2) ? 16 : 8; };
+// units per lane of a dot tile (a tile of w is DU * 32 units; FP64: the warp's sum of a tile
+// and vector is a sixth of its FP64 instructions at 8 units, a tenth at 16)
+template <typename R> struct DotTile { static constexpr int DU = 16; };
 
 }  // namespace
