@@ -250,6 +250,7 @@ void gdr_op_destroy(gdr_op* op) {
   cudaFree(op->rp_off);
   cudaFree(op->nz_off);
   cudaFree(op->nrow);
+  cudaFree(op->tiles);
   cudaFree(op->rowptr);
   cudaFree(op->col);
   cudaFree(op->vals128);

@@ -238,6 +238,8 @@ struct gdr_op {
   long* rp_off = nullptr;
   long* nz_off = nullptr;
   int* nrow = nullptr;
+  int2* tiles = nullptr;  // every 256-row tile of every problem: {problem, tile}
+  long ntiles = 0;
   std::vector<long> nrow_host;
   // Wilson: links stored structure-of-arrays [mu][e][V], e = a*3 + b
   int dims[4] = {0, 0, 0, 0};
