@@ -219,11 +219,84 @@ DEV void warp_givens_qr(c128* A, int lda, int rows, int j0, int cols, int ntot) 
   }
 }
 
+// Householder QR for the reduced solves, which need R and the transformed right-hand sides
+// but no reflectors: R in the upper triangle, what lies below the diagonal is not v.
+//
+// One CTA's FP64 pipe bounds it -- an instruction holds a warp's sub-partition for ~64 cycles
+// whatever its active lanes -- and cta_qr spent most instructions on few lanes: a block sum,
+// divisions by one thread, warp sums of ten additions per column.  Here a reflector is two
+// passes: with x the column below the diagonal, the dots d_c = x^H A[:, c] of all columns
+// (its own gives the norm), each by L lanes (4, 8 or 16, as many as keep all columns in a
+// pass), then, with v = x scal known, A[:, c] -= x (scal f_c), f_c = conj(tau) (A[j, c] +
+// conj(scal) d_c).  The scalars are formed by every thread for itself, two barriers a column.
+// A 41 x 40 system with six shifts (two such solves one after the other): 1,110 us before.
+template <int L>
+DEV double reflect_r(c128* A, int lda, int j, int last, int ntot, double* norm_s) {  // returns R[j, j]
+  const int g = threadIdx.x / L, l = threadIdx.x % L, NG = DT / L;
+  const c128* x = A + (long)j * lda;
+  constexpr int NP = 4;  // passes over the columns: at most GDR_MAX_M + 2 of them, 32 groups or more
+  c128 dc[NP];
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    const int cc = j + g + p * NG;
+    if (j + p * NG >= ntot) break;  // uniform
+    CSum<double> sum;
+    if (cc < ntot) {
+      const c128* col = A + (long)cc * lda;
+      for (int i = j + 1 + l; i <= last; i += L) sum.macc(x[i], col[i]);
+    }
+    c128 v = sum.value();
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) v += shfl_xor_c(v, o);
+    dc[p] = v;
+    if (p == 0 && threadIdx.x == 0) *norm_s = v.x;
+  }
+  __syncthreads();
+  const double s = *norm_s;
+  const c128 alpha = x[j];
+  if (s == 0.0 && alpha.y == 0.0) return alpha.x;  // uniform: nothing to reflect
+  const double n2 = norm2(alpha) + s, inv = rsqrt_nr(n2);
+  const double beta = -copysign(n2 * inv, alpha.x), ib = -copysign(inv, alpha.x);
+  const c128 ctau = {(beta - alpha.x) * ib, alpha.y * ib};  // conj(tau)
+  const c128 ab = {alpha.x - beta, alpha.y};
+  const double rd = 1.0 / norm2(ab);
+  const c128 scal = {ab.x * rd, -ab.y * rd};
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    const int cc = j + g + p * NG;
+    if (j + p * NG >= ntot) break;
+    const bool on = cc < ntot && cc != j;
+    c128* col = A + (long)cc * lda;
+    c128 f = {0, 0};
+    if (on) {
+      f = ctau * cfma(col[j], conj(scal), dc[p]);
+      const c128 h = scal * f;
+      for (int i = j + 1 + l; i <= last; i += L) col[i] = cfnma(col[i], x[i], h);
+    }
+    __syncwarp();  // the group's lanes have read col[j]
+    if (on && l == 0) col[j] -= f;
+  }
+  return beta;
+}
+
+DEV void cta_qr_r(c128* A, int lda, int rows, int cols, int ntot, Sh& sh, int kfull) {
+  for (int j = 0; j < cols && j < rows; ++j) {
+    const int last = qr_last(j, rows, kfull), nc = ntot - j;
+    // two norm slots in turn: a thread may still read this column's while the next is written
+    double* ns = &sh.red[j & 1];
+    const double rjj = nc > DT / 8    ? reflect_r<4>(A, lda, j, last, ntot, ns)
+                       : nc > DT / 16 ? reflect_r<8>(A, lda, j, last, ntot, ns)
+                                      : reflect_r<16>(A, lda, j, last, ntot, ns);
+    __syncthreads();
+    if (threadIdx.x == 0) A[j + (long)j * lda] = {rjj, 0.0};  // no one reads it again before hess_qr's barrier
+  }
+}
+
 // QR of the GMRES recurrence matrix: Householder reflectors for its dense leading
 // block (columns < kfull - 1), Givens rotations for the Hessenberg columns after it.
 DEV void hess_qr(c128* A, int lda, int rows, int cols, int ntot, c128* tau, Sh& sh, int kfull) {
   const int jd = max(0, min(cols, kfull - 1));
-  cta_qr(A, lda, rows, jd, ntot, tau, sh, kfull);
+  cta_qr_r(A, lda, rows, jd, ntot, sh, kfull);
   warp_givens_qr(A, lda, rows, jd, cols, ntot);
   __syncthreads();
 }
@@ -248,7 +321,7 @@ DEV bool fast_backsolve(const c128* A, int lda, int nsz, c128* y, c128* rinv, Sh
       const c128 xj = y[j] * rinv[j];
       __syncwarp();
       if (threadIdx.x == 0) y[j] = xj;
-      for (int i = threadIdx.x; i < j; i += 32) y[i] -= A[i + (long)j * lda] * xj;
+      for (int i = threadIdx.x; i < j; i += 32) y[i] = cfnma(y[i], A[i + (long)j * lda], xj);
       __syncwarp();
     }
   }
@@ -427,7 +500,7 @@ DEV void base_ls(const DenseCycle& d, int c, c128* A, Sh& sh) {
       for (int j = 0; j < me; ++j) {
         c128 hij = H[i + (long)j * (m + 1)];
         if (i == j) hij -= sig;
-        v -= hij * y[j];
+        v = cfnma(v, hij, y[j]);
       }
     }
     s[i] = v;
