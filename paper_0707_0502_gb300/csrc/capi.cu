@@ -31,11 +31,14 @@ gdr_status guarded(gdr_ctx* ctx, F&& f) {
 
 // a tensor-core wait that gave up during the call (the kernel then returned without
 // its result): report it as GDR_ETIMEOUT and clear the flag for the next call
+// (waits for the stream: the flag comes behind the call's kernels, through pinned memory)
 void tc_check(gdr_ctx* ctx) {
-  if (!ctx->tc_err) return;
-  int e = 0;
-  GDR_CUDA(cudaMemcpy(&e, ctx->tc_err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (e) {
+  int* e = static_cast<int*>(ctx->host_status(sizeof(int)));
+  *e = 0;
+  if (ctx->tc_err)
+    GDR_CUDA(cudaMemcpyAsync(e, ctx->tc_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  GDR_CUDA(cudaStreamSynchronize(ctx->stream));
+  if (*e) {
     GDR_CUDA(cudaMemsetAsync(ctx->tc_err, 0, sizeof(int), ctx->stream));
     GDR_CUDA(cudaStreamSynchronize(ctx->stream));
     throw gdr_error(GDR_ETIMEOUT, "tensor-core projection: a wait gave up");
@@ -425,7 +428,6 @@ gdr_status gdr_solve_multishift(gdr_ctx* ctx, const gdr_op* A, int ns, const dou
     else
       result = solve_pipeline<double>(ctx, A, sig, nrhs, Bi, ld, Xi, ld, pr, defl_out, rep);
     stage_out(ctx, A, ns * nrhs, Xi, ld, X, kout);
-    GDR_CUDA(cudaStreamSynchronize(ctx->stream));
     tc_check(ctx);
     rep.t_total_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     rep.kernel_launches = ctx->launches - launches0;
@@ -481,7 +483,6 @@ gdr_status gdr_solve_batch(gdr_ctx* ctx, const gdr_op* A, int ns, const double* 
                                  nq * sizeof(c128), ns, kout, ctx->stream));
       off += nq;
     }
-    GDR_CUDA(cudaStreamSynchronize(ctx->stream));
     tc_check(ctx);
     rep.t_total_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     rep.kernel_launches = ctx->launches - launches0;
@@ -562,7 +563,6 @@ gdr_status gdr_solve_proj(gdr_ctx* ctx, const gdr_op* A, const gdr_defl* defl, i
     else
       run(double{});
     stage_out(ctx, A, ns * nrhs, Xi, ld, X, kout);
-    GDR_CUDA(cudaStreamSynchronize(ctx->stream));
     tc_check(ctx);
     rep.t_total_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     rep.kernel_launches = ctx->launches - launches0;
@@ -934,6 +934,12 @@ gdr_status gdr_basis_dot(gdr_ctx* ctx, gdr_prec prec, long n, int nv, const void
     GDR_REQUIRE(V && R && C, "null argument");
     GDR_CUDA(cudaSetDevice(ctx->device));
     ctx->tc_proj = !(flags & GDR_FLAG_NO_TENSOR_CORES);
+    if (prec != GDR_PREC_FP64 &&
+        gs_dot_tc(ctx, n, nv, static_cast<const c64*>(V), n, ncol, static_cast<const c64*>(R), ldr,
+                  reinterpret_cast<c128*>(C), nv, nullptr, ((double)nv + ncol) * n * sizeof(c64))) {
+      tc_check(ctx);
+      return;
+    }
     auto run = [&](auto zero) {
       using R_ = decltype(zero);
       Batch<R_> b;
@@ -963,7 +969,6 @@ gdr_status gdr_basis_dot(gdr_ctx* ctx, gdr_prec prec, long n, int nv, const void
       gs_dot<R_>(ctx, b, nv, static_cast<const cx<R_>*>(R), ldr, h, false, nullptr);
       GDR_CUDA(cudaMemcpy2DAsync(C, sizeof(c128) * nv, h, sizeof(c128) * (nv + 2), sizeof(c128) * nv, ncol,
                                  cudaMemcpyDeviceToDevice, ctx->stream));
-      GDR_CUDA(cudaStreamSynchronize(ctx->stream));
       tc_check(ctx);
     };
     if (prec == GDR_PREC_FP64)
@@ -981,13 +986,7 @@ gdr_status gdr_basis_residual_update(gdr_ctx* ctx, gdr_prec prec, long n, int nv
     GDR_REQUIRE(V && T && R, "null argument");
     GDR_CUDA(cudaSetDevice(ctx->device));
     ctx->tc_proj = !(flags & GDR_FLAG_NO_TENSOR_CORES);
-    ColState* st = ctx->get<ColState>("bres.st", (size_t)ncol);
-    ColState s0 = {};
-    s0.run = 1;
-    s0.active = 1;
-    std::vector<ColState> sv(ncol, s0);
-    GDR_CUDA(cudaMemcpyAsync(st, sv.data(), sizeof(ColState) * ncol, cudaMemcpyHostToDevice, ctx->stream));
-    gs_dot_shared_reserve(ctx, n, ncol, nv);
+    const ColState* st = nullptr;  // every column
     const c128* Tc = reinterpret_cast<const c128*>(T);
     if (prec == GDR_PREC_FP64)
       combine<double>(ctx, n, ncol, static_cast<c128*>(const_cast<void*>(V)), n, 0, nv, Tc, nv, nv, 0, 0, 2, nullptr,
@@ -995,7 +994,6 @@ gdr_status gdr_basis_residual_update(gdr_ctx* ctx, gdr_prec prec, long n, int nv
     else
       combine<float>(ctx, n, ncol, static_cast<c64*>(const_cast<void*>(V)), n, 0, nv, Tc, nv, nv, 0, 0, 2, nullptr, 0,
                      0, static_cast<c64*>(R), ldr, st);
-    GDR_CUDA(cudaStreamSynchronize(ctx->stream));
     tc_check(ctx);
   });
 }

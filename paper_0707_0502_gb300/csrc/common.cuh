@@ -131,7 +131,8 @@ struct gdr_ctx {
   size_t combine_smem_limit = 0;  // ... and to the basis-combination kernel
   bool tc_ok = false;              // tensor-core projection dot usable (tensor-map encoder, shared memory)
   bool tc_update_ok = false;     // the tensor-core combination kernels fit this device
-  size_t tc_combine_smem = 0;      // dynamic shared memory of the restart's form of them
+  size_t tc_combine_smem = 0;      // ... and the dynamic shared memory they may use
+  size_t tc_dot_smem = 0;          // dynamic shared memory of the projection dot
   bool tc_proj = true;             // use it in this solve (GDR_FLAG_NO_TENSOR_CORES clears it)
   int* tc_err = nullptr;           // set by the tensor-core kernel when a wait timed out
   int sweep_blocks[3] = {0, 0, 0};  // co-resident blocks per SM of the sweep kernel (c64, bf16 links, c128)

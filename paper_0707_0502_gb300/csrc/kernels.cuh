@@ -79,6 +79,10 @@ void gs_dot(gdr_ctx* ctx, const Batch<R>& b, int nv, const cx<R>* w, long wcs, c
 // workspace of gs_dot for ncol columns sharing one basis of nv <= 48 vectors (vcs = 0), to be
 // reserved before a CUDA graph capture that contains such a gs_dot
 void gs_dot_shared_reserve(gdr_ctx* ctx, long n, int ncol, int nv);
+// The tensor-core form of gs_dot alone: out[c * hs + i] = v_i^H r_c for the columns whose state
+// (st, may be null) runs.  False (nothing launched) when it does not apply.
+bool gs_dot_tc(gdr_ctx* ctx, long n, int nv, const c64* V, long ldv, int ncol, const c64* R, long ldr, c128* out,
+               int hs, const ColState* st, double prof_bytes);
 // wout_c = w_c - V_c[:, 0:nv] h_c and h_out[c][0..nv-1] = V_c[:, 0:nv]^H wout_c in one pass
 template <typename R>
 void gs_update_dot(gdr_ctx* ctx, const Batch<R>& b, int nv, const cx<R>* w, cx<R>* wout, long wcs, const c128* h,

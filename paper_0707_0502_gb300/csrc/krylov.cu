@@ -793,15 +793,27 @@ __global__ void __launch_bounds__(DS_W * 32) gs_dot_shared_kernel(long n, const 
   for (int i = lane; i < nv; i += 32) part[((long)slot * ncol + c) * nv + i] = accd[warp * NVM + i];
 }
 
-// hout[c * hs + i] = sum over the S slots of part[(slot * ncol + c) * nv + i] (fixed order)
-__global__ void gs_dot_shared_sum_kernel(int S, int ncol, int nv, const c128* __restrict__ part, c128* hout, int hs,
-                                         const ColState* st) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= ncol * nv) return;
+// hout[c * hs + i] = sum over the S slots of part[(slot * ncol + c) * nv + i]: a block takes 32
+// values, eight warps every eighth slot each (coalesced over the values), their sums added in
+// a fixed order.  One thread per value walking all slots left most of the GPU idle: 16^4, 31
+// vectors x 64 columns, 152 slots: eight blocks, ~40 us.
+__global__ void __launch_bounds__(256) gs_dot_shared_sum_kernel(int S, int ncol, int nv, const c128* __restrict__ part,
+                                                                c128* hout, int hs, const ColState* st) {
+  __shared__ c128 sum[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, tot = ncol * nv;
+  const int t = blockIdx.x * 32 + lane;
+  c128 acc = {0, 0};
+  if (t < tot) {
+#pragma unroll 8
+    for (int q = w; q < S; q += 8) acc += ldcg128(part + (long)q * tot + t);
+  }
+  sum[w][lane] = acc;
+  __syncthreads();
+  if (w != 0 || t >= tot) return;
+#pragma unroll
+  for (int q = 1; q < 8; ++q) acc += sum[q][lane];
   const int c = t / nv, i = t % nv;
   if (st && !st[c].run) return;
-  c128 acc = {0, 0};
-  for (int q = 0; q < S; ++q) acc += part[((long)q * ncol + c) * nv + i];
   hout[(long)c * hs + i] = acc;
 }
 
@@ -916,26 +928,29 @@ static void gs_dot_shared_launch(gdr_ctx* ctx, const Batch<R>& b, int nv, const 
     GDR_LAUNCHED(ctx);
   }
   const int tot = b.ncol * nv;
-  gs_dot_shared_sum_kernel<<<(tot + 255) / 256, 256, 0, ctx->stream>>>(S, b.ncol, nv, part, h_out, b.m + 2, b.st);
+  gs_dot_shared_sum_kernel<<<(tot + 31) / 32, 256, 0, ctx->stream>>>(S, b.ncol, nv, part, h_out, b.m + 2, b.st);
   GDR_LAUNCHED(ctx);
+}
+
+bool gs_dot_tc(gdr_ctx* ctx, long n, int nv, const c64* V, long ldv, int ncol, const c64* R, long ldr, c128* out,
+               int hs, const ColState* st, double prof_bytes) {
+  if (ncol < TC_MIN_COLS || !ctx->tc_ok || !ctx->tc_proj || !ctx->tc_err) return false;
+  c128* part = ctx->get<c128>("dsh.part", (size_t)tc_proj_splits(ctx, n, ncol) * ncol * nv + 64);
+  int S = 0;
+  if (!tc_proj_dot(ctx, n, V, ldv, nv, R, ldr, ncol, part, ctx->tc_err, S, prof_bytes)) return false;
+  const int tot = ncol * nv;
+  gs_dot_shared_sum_kernel<<<(tot + 31) / 32, 256, 0, ctx->stream>>>(S, ncol, nv, part, out, hs, st);
+  GDR_LAUNCHED(ctx);
+  return true;
 }
 
 template <typename R>
 void gs_dot(gdr_ctx* ctx, const Batch<R>& b, int nv, const cx<R>* w, long wcs, c128* h_out, bool wnorm,
             const cx<R>* wprev) {
-  if (std::is_same<R, float>::value && b.vcs == 0 && b.ncol >= TC_MIN_COLS && b.nvec == nullptr && !wnorm &&
-      !wprev && ctx->tc_ok && ctx->tc_proj && ctx->tc_err) {  // tensor cores
-    const int S0 = tc_proj_splits(ctx, b.n, b.ncol);
-    c128* part = ctx->get<c128>("dsh.part", (size_t)S0 * b.ncol * nv + 64);
-    int S = 0;
-    const double bytes = ctx->profile ? ((double)nv * b.n + col_len(b)) * sizeof(cx<R>) * run_share(ctx, b) : 0.0;
-    if (tc_proj_dot(ctx, b.n, reinterpret_cast<const c64*>(b.V), b.ldv, nv, reinterpret_cast<const c64*>(w), wcs,
-                    b.ncol, part, ctx->tc_err, S, bytes)) {
-      const int tot = b.ncol * nv;
-      gs_dot_shared_sum_kernel<<<(tot + 255) / 256, 256, 0, ctx->stream>>>(S, b.ncol, nv, part, h_out, b.m + 2,
-                                                                           b.st);
-      GDR_LAUNCHED(ctx);
-      return;
+  if constexpr (std::is_same<R, float>::value) {
+    if (b.vcs == 0 && b.nvec == nullptr && !wnorm && !wprev) {
+      const double bytes = ctx->profile ? ((double)nv * b.n + col_len(b)) * sizeof(cx<R>) * run_share(ctx, b) : 0.0;
+      if (gs_dot_tc(ctx, b.n, nv, b.V, b.ldv, b.ncol, w, wcs, h_out, b.m + 2, b.st, bytes)) return;
     }
   }
   if (dot_shared_applies(b, nv, wnorm, wprev)) {  // one basis for many columns: read it once

@@ -40,12 +40,13 @@ namespace {
 
 constexpr int TC_M = 128;      // MMA rows: basis vectors, zero-filled above nv
 constexpr int TC_KF = 32;      // floats per K stage: one 128-byte swizzle row
-constexpr int TC_STAGES = 4;
+constexpr int TC_MAXST = 8;    // stages of the ring
 constexpr int TC_THREADS = 256;  // warp 0 TMA, warp 1 MMA, warp 2 tensor-memory owner, warps 4-7 prime + epilogue
 constexpr unsigned TC_A_BYTES = TC_M * TC_KF * 4;  // 16 KB
 
 struct TcArgs {
   int ncol, nv, nt;      // columns, basis vectors, MMA N (multiple of 16, <= 128)
+  int nst;               // stages
   long ksteps;           // K stages of the whole vector (2n / 32 rounded up)
   long ksplit;           // K stages per CTA
   c128* part;            // [K range][ncol][nv] FP64 partials
@@ -138,34 +139,42 @@ DEV void tmem_ld16(uint32_t t, float (&v)[16]) {
 }
 
 // accumulator layout in tensor memory: D_re in columns [0, nt), D_im from column im_off
+// (STACK: D_re and D_im in the two halves of the rows, one accumulator)
 HD int tc_im_off(int nt) { return (nt + 31) / 32 * 32; }
-HD uint32_t tc_cols(int nt) {
-  const int need = 2 * tc_im_off(nt);
+HD uint32_t tc_cols(int nt, bool stack) {
+  const int need = (stack ? 1 : 2) * tc_im_off(nt);
   return need <= 32 ? 32u : need <= 64 ? 64u : need <= 128 ? 128u : 256u;
 }
+HD unsigned tc_stage_bytes(int nt, bool stack) { return (stack ? 1u : 2u) * TC_A_BYTES + (unsigned)nt * TC_KF * 4; }
 
+// STACK (nv <= 64): rows 0..63 of one operand are V, rows 64..127 V', so a stage is four MMAs
+// (issuing one takes a thread ~80 cycles, and a stage of 31 vectors and 64 columns is ~550
+// cycles of HBM time: eight MMAs a stage were slower than HBM), 8 KB to bring and only nv
+// rows to prime, and the ring holds up to eight stages instead of four.
+template <bool STACK>
 __global__ void __launch_bounds__(TC_THREADS, 1) tc_proj_dot_kernel(const __grid_constant__ CUtensorMap mapV,
                                                                    const __grid_constant__ CUtensorMap mapR,
                                                                    TcArgs a) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  constexpr unsigned V_BYTES = STACK ? TC_A_BYTES / 2 : TC_A_BYTES;  // V's tile, V' right behind it
   const unsigned b_bytes = (unsigned)a.nt * TC_KF * 4;
-  const unsigned stage_bytes = 2 * TC_A_BYTES + b_bytes;  // V, V', R
-  __shared__ __align__(8) uint64_t full[TC_STAGES], primed[TC_STAGES], empty[TC_STAGES], accb;
+  const unsigned stage_bytes = tc_stage_bytes(a.nt, STACK);  // V, V', R
+  __shared__ __align__(8) uint64_t full[TC_MAXST], primed[TC_MAXST], empty[TC_MAXST], accb;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_s;
   __shared__ long issued_s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long k0 = (long)blockIdx.x * a.ksplit;
-  const long nk = min(a.ksteps, k0 + a.ksplit) - k0;
+  const int nk = (int)(min(a.ksteps, k0 + a.ksplit) - k0);
   const int col0 = blockIdx.y * a.nt;
   const int im_off = tc_im_off(a.nt);
-  const uint32_t tcols = tc_cols(a.nt);
+  const uint32_t tcols = tc_cols(a.nt, STACK);
   if (threadIdx.x == 0) {
-    for (int s = 0; s < TC_STAGES; ++s) {
+    for (int s = 0; s < a.nst; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&primed[s], 128);
+      mbar_init(&primed[s], 4);  // one arrival per warp
       mbar_init(&empty[s], 1);
     }
     mbar_init(&accb, 1);
@@ -179,6 +188,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_proj_dot_kernel(const __grid
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // rows of V' that are never primed
+  for (int s = 0; s < a.nst; ++s) {
+    float4* z = reinterpret_cast<float4*>(base + (size_t)s * stage_bytes + V_BYTES);
+    for (unsigned q = a.nv * 8 + threadIdx.x; q < V_BYTES / 16; q += TC_THREADS) z[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -186,52 +201,64 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_proj_dot_kernel(const __grid
   volatile int* abort = &abort_s;
 
   if (warp == 0 && lane == 0) {  // ---- TMA producer
-    long issued = 0;
-    for (long it = 0; it < nk && !*abort; ++it) {
-      const int s = (int)(it % TC_STAGES);
-      const unsigned ph = (unsigned)((it / TC_STAGES) & 1);
-      if (it >= TC_STAGES && !mbar_wait(&empty[s], ph ^ 1u, abort)) break;
+    int issued = 0, s = 0;
+    unsigned ph = 0;
+    for (int it = 0; it < nk && !*abort; ++it) {
+      if (it >= a.nst && !mbar_wait(&empty[s], ph ^ 1u, abort)) break;
       unsigned char* st = base + (size_t)s * stage_bytes;
-      mbar_arrive_tx(&full[s], TC_A_BYTES + b_bytes);
+      mbar_arrive_tx(&full[s], V_BYTES + b_bytes);
       const int x = (int)((k0 + it) * TC_KF);  // a multiple of 32 floats: 128-byte aligned
       tma_load_2d(st, &mapV, x, 0, &full[s]);
-      tma_load_2d(st + 2 * TC_A_BYTES, &mapR, x, col0, &full[s]);
+      tma_load_2d(st + 2 * V_BYTES, &mapR, x, col0, &full[s]);
       issued = it + 1;
+      if (++s == a.nst) {
+        s = 0;
+        ph ^= 1u;
+      }
     }
     issued_s = issued;
   } else if (warp == 1 && lane == 0) {  // ---- MMA issuer
     const uint32_t idesc = instr_desc(a.nt);
-    for (long it = 0; it < nk; ++it) {
-      const int s = (int)(it % TC_STAGES);
-      const unsigned ph = (unsigned)((it / TC_STAGES) & 1);
+    int s = 0;
+    unsigned ph = 0;
+    for (int it = 0; it < nk; ++it) {
       if (!mbar_wait(&full[s], ph, abort) || !mbar_wait(&primed[s], ph, abort)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       unsigned char* st = base + (size_t)s * stage_bytes;
-      const uint64_t dv = sm_desc(st), dp = sm_desc(st + TC_A_BYTES), dr = sm_desc(st + 2 * TC_A_BYTES);
+      const uint64_t dv = sm_desc(st), dp = dv + (V_BYTES >> 4), dr = dv + (2 * V_BYTES >> 4);
 #pragma unroll
       for (int kk = 0; kk < TC_KF / 8; ++kk) {  // 8 TF32 (32 bytes) per MMA
         const uint32_t acc = (it > 0 || kk > 0) ? 1u : 0u;
         mma_tf32(tm, dv + 2 * kk, dr + 2 * kk, idesc, acc);
-        mma_tf32(tm + (uint32_t)im_off, dp + 2 * kk, dr + 2 * kk, idesc, acc);
+        if (!STACK) mma_tf32(tm + (uint32_t)im_off, dp + 2 * kk, dr + 2 * kk, idesc, acc);
       }
       mma_commit(&empty[s]);
+      if (++s == a.nst) {
+        s = 0;
+        ph ^= 1u;
+      }
     }
     mma_commit(&accb);  // arrives once every MMA issued above has completed
   } else if (warp >= 4) {  // ---- V' = V with (re, im) -> (-im, re), then the epilogue
-    const int t = threadIdx.x - 128;
-    for (long it = 0; it < nk; ++it) {
-      const int s = (int)(it % TC_STAGES);
-      const unsigned ph = (unsigned)((it / TC_STAGES) & 1);
-      if (!mbar_wait(&full[s], ph, abort)) break;
+    const unsigned t = threadIdx.x - 128;
+    int s = 0;
+    unsigned ph = 0;
+    for (int it = 0; it < nk; ++it) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&full[s], ph, abort))) break;
       unsigned char* st = base + (size_t)s * stage_bytes;
       const float4* src = reinterpret_cast<const float4*>(st);
-      float4* dst = reinterpret_cast<float4*>(st + TC_A_BYTES);
-      for (unsigned q = t; q < TC_A_BYTES / 16; q += 128) {
+      float4* dst = reinterpret_cast<float4*>(st + V_BYTES);
+      for (unsigned q = t; q < (unsigned)a.nv * 8; q += 128) {
         const float4 v = src[q];
         dst[q] = make_float4(-v.y, v.x, -v.w, v.z);
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      mbar_arrive(&primed[s]);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&primed[s]);
+      if (++s == a.nst) {
+        s = 0;
+        ph ^= 1u;
+      }
     }
     // the MMAs finish (or time out) before the accumulators are read or freed; this
     // wait does not follow the CTA's abort flag
@@ -243,18 +270,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_proj_dot_kernel(const __grid
     if (__all_sync(0xffffffffu, got && !*abort)) {
       // accumulators: tensor-memory lane = basis vector, column = matrix column
       const int q4 = warp & 3;
-      const int row = q4 * 32 + lane;
       const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
       for (int cb = 0; cb < a.nt; cb += 32) {
         float re[32], im[32];
         tmem_ld32(tm + lane_base + (uint32_t)cb, re);
-        tmem_ld32(tm + lane_base + (uint32_t)(im_off + cb), im);
+        if (!STACK) tmem_ld32(tm + lane_base + (uint32_t)(im_off + cb), im);
+        const int row = STACK ? (q4 & 1) * 32 + lane : q4 * 32 + lane;
         if (row < a.nv) {
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             const int c = col0 + cb + j;
-            if (cb + j < a.nt && c < a.ncol)
-              a.part[((long)blockIdx.x * a.ncol + c) * a.nv + row] = c128{(double)re[j], (double)im[j]};
+            if (cb + j >= a.nt || c >= a.ncol) continue;
+            c128* p = &a.part[((long)blockIdx.x * a.ncol + c) * a.nv + row];
+            if (STACK) (q4 < 2 ? p->x : p->y) = (double)re[j];
+            else *p = c128{(double)re[j], (double)im[j]};
           }
         }
       }
@@ -266,9 +295,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_proj_dot_kernel(const __grid
     // wait (bounded) for the last load issued into each stage, then report the failure
     if (warp == 0 && lane == 0) {
       const long issued = issued_s;
-      for (long it = issued > TC_STAGES ? issued - TC_STAGES : 0; it < issued; ++it) {
+      for (long it = issued > a.nst ? issued - a.nst : 0; it < issued; ++it) {
         int own = 0;
-        mbar_wait(&full[(int)(it % TC_STAGES)], (unsigned)((it / TC_STAGES) & 1), &own);
+        mbar_wait(&full[(int)(it % a.nst)], (unsigned)((it / a.nst) & 1), &own);
       }
       atomicExch(a.err, 1);
     }
@@ -783,8 +812,6 @@ bool make_map_raw(CUtensorMap& m, const void* ptr, long n, long ld, int rows, lo
 
 }  // namespace
 
-size_t tc_proj_smem(int nt) { return 1024 + (size_t)TC_STAGES * (2 * TC_A_BYTES + (size_t)nt * TC_KF * 4); }
-
 int tc_proj_splits(gdr_ctx* ctx, long n, int ncol) {
   const int ctiles = (ncol + 127) / 128;
   const long ksteps = (2 * n + TC_KF - 1) / TC_KF;
@@ -799,8 +826,9 @@ bool tc_proj_dot(gdr_ctx* ctx, long n, const c64* V, long ldv, int nv, const c64
   const int ctiles = (ncol + 127) / 128;
   const int per = (ncol + ctiles - 1) / ctiles;
   const int nt = std::max(16, (per + 15) / 16 * 16);
+  const bool stack = nv <= TC_M / 2;
   CUtensorMap mv, mr;
-  if (!make_map(mv, V, n, ldv, nv, TC_M) || !make_map(mr, R, n, ldr, ncol, nt)) return false;
+  if (!make_map(mv, V, n, ldv, nv, stack ? TC_M / 2 : TC_M) || !make_map(mr, R, n, ldr, ncol, nt)) return false;
   TcArgs a;
   a.ncol = ncol;
   a.nv = nv;
@@ -810,10 +838,13 @@ bool tc_proj_dot(gdr_ctx* ctx, long n, const c64* V, long ldv, int nv, const c64
   a.ksplit = (a.ksteps + nsplit - 1) / nsplit;
   a.part = part;
   a.err = err;
-  const size_t smem = tc_proj_smem(nt);
+  const size_t sb = tc_stage_bytes(nt, stack);
+  a.nst = (int)std::min<size_t>(TC_MAXST, (ctx->tc_dot_smem - 1024) / sb);
+  const size_t smem = 1024 + a.nst * sb;
   dim3 grid((unsigned)nsplit, (unsigned)ctiles);
   KProf kp(ctx, "tc_proj_dot_c64", prof_bytes);
-  tc_proj_dot_kernel<<<grid, TC_THREADS, smem, ctx->stream>>>(mv, mr, a);
+  if (stack) tc_proj_dot_kernel<true><<<grid, TC_THREADS, smem, ctx->stream>>>(mv, mr, a);
+  else tc_proj_dot_kernel<false><<<grid, TC_THREADS, smem, ctx->stream>>>(mv, mr, a);
   GDR_LAUNCHED(ctx);
   return true;
 }
@@ -913,18 +944,15 @@ void tc_proj_init(gdr_ctx* ctx) {
   ctx->tc_ok = false;
   if (!encoder()) return;
   cudaFuncAttributes at;
-  if (cudaFuncGetAttributes(&at, tc_proj_dot_kernel) != cudaSuccess) return;
-  const size_t need = tc_proj_smem(128);
-  if (need + at.sharedSizeBytes > ctx->max_smem_optin) return;
-  if (cudaFuncSetAttribute(tc_proj_dot_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need) != cudaSuccess)
-    return;
-  ctx->tc_ok = true;
-  ctx->tc_update_ok = false;
   auto allow = [&](auto kernel) {  // dynamic shared memory this kernel may use
     if (cudaFuncGetAttributes(&at, kernel) != cudaSuccess || at.sharedSizeBytes >= ctx->max_smem_optin) return (size_t)0;
     const size_t dyn = ctx->max_smem_optin - at.sharedSizeBytes;
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) == cudaSuccess ? dyn : 0;
   };
+  ctx->tc_dot_smem = std::min(allow(tc_proj_dot_kernel<true>), allow(tc_proj_dot_kernel<false>));
+  if (ctx->tc_dot_smem < 1024 + 3 * (size_t)tc_stage_bytes(128, false)) return;
+  ctx->tc_ok = true;
+  ctx->tc_update_ok = false;
   const int ka = (2 * TU_MAXNV + 31) / 32;
   ctx->tc_combine_smem = std::min({allow(tc_combine_kernel<TU_RESTART>), allow(tc_combine_kernel<TU_DIRECT>),
                                    allow(tc_combine_kernel<TU_REDUCE>)});
