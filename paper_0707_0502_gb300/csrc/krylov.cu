@@ -445,22 +445,33 @@ __global__ void __launch_bounds__(NT) norms2_kernel(long n, const T* __restrict_
   // <= 8 * 2^-24 per group) and only the group sums in FP64: the FP64 pipe, slow on this
   // part, would otherwise bound the kernel.  FP64 vectors are summed in FP64 throughout.
   double s = 0;
-  long i = blockIdx.x * (long)NT + threadIdx.x;
-  const long stride = (long)gridDim.x * NT;
+  const long nu = nunits<R>(n), stride = (long)gridDim.x * NT;
+  constexpr int K = U<R>::K;
   if (sizeof(R) == 4) {
-    for (; i + 3 * stride < n; i += 4 * stride) {
-      T v[4];
+    for (long u = blockIdx.x * (long)NT + threadIdx.x; u < nu; u += 4 * stride) {  // four 16-byte units in flight
+      T v[4][K];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) v[q] = xc[i + q * stride];
-      float f = 0.f;
+      for (int q = 0; q < 4; ++q) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) f = fmaf((float)v[q].x, (float)v[q].x, fmaf((float)v[q].y, (float)v[q].y, f));
-      s += (double)f;
+        for (int kk = 0; kk < K; ++kk) v[q][kk] = {0, 0};
+        if (u + q * stride < nu) ldu<R>(xc, u + q * stride, n, v[q]);
+      }
+#pragma unroll
+      for (int h = 0; h < 4; h += 2) {
+        float f = 0.f;
+#pragma unroll
+        for (int q = h; q < h + 2; ++q)
+#pragma unroll
+          for (int kk = 0; kk < K; ++kk)
+            f = fmaf((float)v[q][kk].x, (float)v[q][kk].x, fmaf((float)v[q][kk].y, (float)v[q][kk].y, f));
+        s += (double)f;
+      }
     }
-  }
-  for (; i < n; i += stride) {
-    const T v = xc[i];
-    s = fma((double)v.y, (double)v.y, fma((double)v.x, (double)v.x, s));
+  } else {
+    for (long i = blockIdx.x * (long)NT + threadIdx.x; i < n; i += stride) {
+      const T v = xc[i];
+      s = fma((double)v.y, (double)v.y, fma((double)v.x, (double)v.x, s));
+    }
   }
   c128 d[1] = {{s, 0}};
   block_reduce<double, 1>(d, part + (long)c * gridDim.x + blockIdx.x, 1);
@@ -1037,6 +1048,10 @@ void start_cycle(gdr_ctx* ctx, const Batch<R>& b, const cx<R>* r, long rcs) {
 template <typename T>
 void norms2(gdr_ctx* ctx, long n, int cols, const T* x, long xcs, double* out, c128* part, int nblk, unsigned* cnt,
             const int* nvec) {
+  // enough blocks for the GPU, no more than give each thread a round of loads (16^4, 64 columns:
+  // 456 blocks a column, the most the partials allow, left 1.7 elements of each round of four)
+  const long want = std::max<long>((8L * ctx->num_sms + cols - 1) / cols, (n * (long)sizeof(T) / 16 + 4 * NT - 1) / (4 * NT) / 4);
+  nblk = (int)std::max<long>(1, std::min<long>(nblk, want));
   dim3 grid((unsigned)nblk, (unsigned)cols);
   KProf kp(ctx, sizeof(T) == 8 ? "norms_c64" : "norms_c128", (double)n * sizeof(T) * cols);
   norms2_kernel<T><<<grid, NT, 0, ctx->stream>>>(n, x, xcs, out, part, cnt, nvec);
