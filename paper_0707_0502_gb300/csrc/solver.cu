@@ -428,6 +428,19 @@ std::vector<ColState> read_states(gdr_ctx* ctx, const ColState* st, int ncol) {
   return std::vector<ColState>(h, h + ncol);
 }
 
+// Persistent sweep or one launch per phase for the Arnoldi steps of a stage: what the
+// autotuner chose, else launches, except for a single FP64 column of at most 1,024 elements.
+// A pass of 20 steps in ms, sweep / launches: complex64 4^4 0.53 / 0.34, 8^4 0.67 / 0.39, six
+// columns of 8^4 1.23 / 0.55; FP64 4^4 1.15 / 1.06, 8^4 2.43 / 1.45, n = 1,000 (25 steps) 1.03 /
+// 1.11, n = 384 0.94 / 0.97.
+template <typename R>
+bool use_sweep(gdr_ctx* ctx, const gdr_op* A, const Batch<R>& b) {
+  if (!sweep_fits<R>(ctx, A, b)) return false;
+  const int tuned = sweep_choice(A, std::is_same<R, double>::value, b.ncol, b.m);
+  if (tuned >= 0) return tuned != 0;
+  return std::is_same<R, double>::value && b.ncol == 1 && b.n <= 1024;
+}
+
 }  // namespace
 
 // ------------------------------------------------------------- GMRES-DR-Sh
@@ -473,8 +486,7 @@ DrResult dr_sh(gdr_ctx* ctx, const gdr_op* A, const DrJob<R>& job, bool use_grap
   GDR_LAUNCHED(ctx);
   start_cycle<R>(ctx, b, job.rhs, job.ldrhs);
 
-  const bool sweep = job.sweep && sweep_fits<R>(ctx, A, b) &&
-                    sweep_choice(A, std::is_same<R, double>::value, ncol, m) != 0;
+  const bool sweep = job.sweep && use_sweep<R>(ctx, A, b);
   if (sweep) sweep_reserve<R>(ctx, b);
   Graph g_first, g_next;
   DrResult res;
@@ -696,8 +708,7 @@ ProjResult proj_batch(gdr_ctx* ctx, const gdr_op* A, const ProjJob<R>& job, bool
   d.want_r = true;
   d.ls32 = std::is_same<R, float>::value && job.ls32;  // GMRES(m_p) cycles on a complex64 basis
 
-  const bool sweep = job.sweep && sweep_fits<R>(ctx, A, b) &&
-                    sweep_choice(A, std::is_same<R, double>::value, ncol, mp) != 0;
+  const bool sweep = job.sweep && use_sweep<R>(ctx, A, b);
   if (sweep) sweep_reserve<R>(ctx, b);
   Graph gr;
   ProjResult res;
