@@ -190,6 +190,7 @@ __global__ void __launch_bounds__(NT, wilson_min_blocks<R>(NT)) wilson_kernel(co
   int c;
   tile_col(ncol, col_inner, tile, c);
   long site = tile * NT + threadIdx.x;
+  pdl_wait();
   if (run && !run[(long)c * run_stride]) return;
   if (site >= V) {  // a warp that stores together keeps all its lanes
     if (!out_sm || (site & ~31L) >= V) return;
@@ -268,6 +269,7 @@ __global__ void __launch_bounds__(128) wilson_split_kernel(const LT* __restrict_
   long tile;
   int c;
   tile_col(ncol, col_inner, tile, c);
+  pdl_wait();
   if (run && !run[(long)c * run_stride]) return;
   const int mu = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long site0 = tile * 32L, site = site0 + lane;
@@ -324,6 +326,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) wilson_pair_kernel(
   int cp;
   tile_col(npair, col_inner, tile, cp);
   long site = tile * NT + threadIdx.x;
+  pdl_wait();
   if (site >= V) {
     if (!out_sm || (site & ~31L) >= V) return;
     site = V - 1;
@@ -519,7 +522,7 @@ static void wilson_launch(gdr_ctx* ctx, const gdr_op* A, const LT* links, const 
     if (s.form == 2) {  // column pairs, packed FP32x2
       const int npair = (ncol + 1) / 2;
 #define GDR_WILSON_PAIR(NT)                                                                                          \
-  wilson_pair_kernel<LT, NT><<<tile_grid((A->V + NT - 1) / NT, npair, s.col_inner), NT, stage(NT), ctx->stream>>>( \
+  launch_pdl(out_sm != 0, wilson_pair_kernel<LT, NT>, tile_grid((A->V + NT - 1) / NT, npair, s.col_inner), NT, stage(NT), ctx->stream, \
       links, d[0], d[1], d[2], d[3], A->diag_a, sigma, X, ldx, Y, ldy, B, ldb, run, run_stride, cpp, xs, xs_stride, \
       ncol, s.col_inner, out_sm)
       if (s.threads == 64) GDR_WILSON_PAIR(64);
@@ -530,12 +533,12 @@ static void wilson_launch(gdr_ctx* ctx, const gdr_op* A, const LT* links, const 
     }
   }
   if (s.form == 1) {
-    wilson_split_kernel<R, LT><<<tile_grid((A->V + 31) / 32, ncol, s.col_inner), 128, 0, ctx->stream>>>(
+    launch_pdl(out_sm != 0, wilson_split_kernel<R, LT>, tile_grid((A->V + 31) / 32, ncol, s.col_inner), 128, 0, ctx->stream,
         links, d[0], d[1], d[2], d[3], A->diag_a, sigma, X, ldx, Y, ldy, B, ldb, run, run_stride, cpp, xs, xs_stride,
         ncol, s.col_inner, out_sm);
   } else {
 #define GDR_WILSON_SITE(NT)                                                                                         \
-  wilson_kernel<R, LT, NT><<<tile_grid((A->V + NT - 1) / NT, ncol, s.col_inner), NT, stage(NT), ctx->stream>>>(     \
+  launch_pdl(out_sm != 0, wilson_kernel<R, LT, NT>, tile_grid((A->V + NT - 1) / NT, ncol, s.col_inner), NT, stage(NT), ctx->stream, \
       links, d[0], d[1], d[2], d[3], A->diag_a, sigma, X, ldx, Y, ldy, B, ldb, run, run_stride, cpp, xs, xs_stride, \
       ncol, s.col_inner, out_sm)
     if (s.threads == 64) GDR_WILSON_SITE(64);
