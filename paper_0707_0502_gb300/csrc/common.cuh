@@ -128,6 +128,7 @@ struct gdr_ctx {
   size_t max_smem_optin = 0;
   size_t l2_bytes = 0;
   size_t dense_smem_limit = 0;    // dynamic shared memory available to the dense kernels
+  bool dense_cluster = false;     // clusters of the reduced solve can be resident
   size_t combine_smem_limit = 0;  // ... and to the basis-combination kernel
   bool tc_ok = false;              // tensor-core projection dot usable (tensor-map encoder, shared memory)
   bool tc_update_ok = false;     // the tensor-core combination kernels fit this device

@@ -231,7 +231,7 @@ DEV void warp_givens_qr(c128* A, int lda, int rows, int j0, int cols, int ntot) 
 // conj(scal) d_c).  The scalars are formed by every thread for itself, two barriers a column.
 // A 41 x 40 system with six shifts (two such solves one after the other): 1,110 us before.
 template <int L>
-DEV double reflect_r(c128* A, int lda, int j, int last, int ntot, double* norm_s) {  // returns R[j, j]
+DEV double reflect_r(c128* A, int lda, int j, int last, int ntot, double* norm_s, c128* keep) {  // returns R[j, j]
   const int g = threadIdx.x / L, l = threadIdx.x % L, NG = DT / L;
   const c128* x = A + (long)j * lda;
   constexpr int NP = 4;  // passes over the columns: at most GDR_MAX_M + 2 of them, 32 groups or more
@@ -254,13 +254,20 @@ DEV double reflect_r(c128* A, int lda, int j, int last, int ntot, double* norm_s
   __syncthreads();
   const double s = *norm_s;
   const c128 alpha = x[j];
-  if (s == 0.0 && alpha.y == 0.0) return alpha.x;  // uniform: nothing to reflect
+  if (s == 0.0 && alpha.y == 0.0) {  // uniform: nothing to reflect
+    if (keep && threadIdx.x == 0) keep[0] = keep[1] = {0, 0};
+    return alpha.x;
+  }
   const double n2 = norm2(alpha) + s, inv = rsqrt_nr(n2);
   const double beta = -copysign(n2 * inv, alpha.x), ib = -copysign(inv, alpha.x);
   const c128 ctau = {(beta - alpha.x) * ib, alpha.y * ib};  // conj(tau)
   const c128 ab = {alpha.x - beta, alpha.y};
   const double rd = 1.0 / norm2(ab);
   const c128 scal = {ab.x * rd, -ab.y * rd};
+  if (keep && threadIdx.x == 0) {
+    keep[0] = ctau;
+    keep[1] = scal;
+  }
 #pragma unroll
   for (int p = 0; p < NP; ++p) {
     const int cc = j + g + p * NG;
@@ -279,16 +286,55 @@ DEV double reflect_r(c128* A, int lda, int j, int last, int ntot, double* norm_s
   return beta;
 }
 
-DEV void cta_qr_r(c128* A, int lda, int rows, int cols, int ntot, Sh& sh, int kfull) {
+// keep (may be null): conj(tau) and scal of every column, for apply_kept
+DEV void cta_qr_r(c128* A, int lda, int rows, int cols, int ntot, Sh& sh, int kfull, c128* keep = nullptr) {
   for (int j = 0; j < cols && j < rows; ++j) {
     const int last = qr_last(j, rows, kfull), nc = ntot - j;
     // two norm slots in turn: a thread may still read this column's while the next is written
     double* ns = &sh.red[j & 1];
-    const double rjj = nc > DT / 8    ? reflect_r<4>(A, lda, j, last, ntot, ns)
-                       : nc > DT / 16 ? reflect_r<8>(A, lda, j, last, ntot, ns)
-                                      : reflect_r<16>(A, lda, j, last, ntot, ns);
+    c128* kj = keep ? keep + 2 * j : nullptr;
+    const double rjj = nc > DT / 8    ? reflect_r<4>(A, lda, j, last, ntot, ns, kj)
+                       : nc > DT / 16 ? reflect_r<8>(A, lda, j, last, ntot, ns, kj)
+                                      : reflect_r<16>(A, lda, j, last, ntot, ns, kj);
     __syncthreads();
     if (threadIdx.x == 0) A[j + (long)j * lda] = {rjj, 0.0};  // no one reads it again before hess_qr's barrier
+  }
+}
+
+// v <- Q^H v for the reflectors that cta_qr_r kept (x below A's diagonal), v in one warp's
+// registers (rows lane + 32 q, at most 97): one chain of ~35 FP64 instructions per column,
+// no barriers.
+DEV void apply_kept(const c128* A, int lda, int rows, int cols, int kfull, const c128* keep, c128 (&v)[4]) {
+  const int lane = threadIdx.x & 31;
+  for (int j = 0; j < cols && j < rows; ++j) {
+    const int last = qr_last(j, rows, kfull);
+    const c128 *x = A + (long)j * lda, ctau = keep[2 * j], scal = keep[2 * j + 1];
+    CSum<double> sum;
+    c128 vj = {0, 0}, xi[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (32 * q > last) break;  // uniform
+      const int i = lane + 32 * q;
+      xi[q] = (i > j && i <= last) ? x[i] : c128{0, 0};
+      sum.macc(xi[q], v[q]);
+      if (q == j >> 5) vj = v[q];
+    }
+    // both parts over the warp, the first exchange splitting them over its halves
+    const c128 a = sum.value();
+    const bool h = lane & 16;
+    double t = (h ? a.y : a.x) + __shfl_xor_sync(FULL, h ? a.x : a.y, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
+    const c128 d = {__shfl_sync(FULL, t, 0), __shfl_sync(FULL, t, 16)};
+    vj = {__shfl_sync(FULL, vj.x, j & 31), __shfl_sync(FULL, vj.y, j & 31)};
+    const c128 f = ctau * cfma(vj, conj(scal), d);
+    const c128 g = scal * f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (32 * q > last) break;
+      v[q] = cfnma(v[q], xi[q], g);
+      if (lane + 32 * q == j) v[q] -= f;
+    }
   }
 }
 
@@ -515,6 +561,32 @@ DEV void base_ls(const DenseCycle& d, int c, c128* A, Sh& sh) {
   }
 }
 
+// beta_new and d_i from the factored [(Hbar - sigma_i Ibar) | c | s]
+DEV void shift_finish(const DenseCycle& d, int c, int i, c128* A, int lda, c128 beta, c128* y, c128* rinv, Sh& sh) {
+  ColState* st = d.st + c;
+  const int m = d.m, me = st->m_eff, col = (d.k > 0 ? d.k + 1 : 0) + i;
+  const bool broke = st->broke;
+  c128* Cf = d.Cf + (long)c * d.ccs;
+  c128 bnew = {0, 0};
+  if (!broke) {
+    const c128 qc = A[me + (long)me * lda], qs = A[me + (long)(me + 1) * lda];
+    if (qs.x == 0.0 && qs.y == 0.0) {
+      set_err(st, GDR_EBREAKDOWN);
+    } else {
+      bnew = beta * cdiv(qc, qs);
+    }
+  }
+  for (int r = threadIdx.x; r < me; r += DT)
+    y[r] = beta * A[r + (long)me * lda] - bnew * A[r + (long)(me + 1) * lda];
+  __syncthreads();
+  if (!fast_backsolve(A, lda, me, y, rinv, sh)) set_err(st, GDR_EBREAKDOWN);
+  for (int r = threadIdx.x; r <= m; r += DT) Cf[r + (long)col * d.ldc] = (r < me) ? y[r] : c128{0, 0};
+  if (threadIdx.x == 0) {
+    d.beta[(long)c * d.ns + i] = bnew;
+    d.norms[(long)c * d.ns + i] = cabs_(bnew) * st->rnorm;
+  }
+}
+
 // shift i >= 1: [(Hbar - sigma_i Ibar) | c | s] -> QR, beta_new, d_i into Cf column k+1+i
 DEV void shift_solve(const DenseCycle& d, int c, int i, c128* A, Sh& sh) {
   ColState* st = d.st + c;
@@ -577,24 +649,64 @@ DEV void shift_solve(const DenseCycle& d, int c, int i, c128* A, Sh& sh) {
   if (threadIdx.x == 0) sh.ibc[0] = 0;
   __syncthreads();
   hess_qr(A, lda, rows, me, me + 2, tau, sh, d.kfull);
-  c128 bnew = {0, 0};
-  if (!broke) {
-    const c128 qc = A[me + (long)me * lda], qs = A[me + (long)(me + 1) * lda];
-    if (qs.x == 0.0 && qs.y == 0.0) {
-      set_err(st, GDR_EBREAKDOWN);
-    } else {
-      bnew = beta * cdiv(qc, qs);
+  shift_finish(d, c, i, A, lda, beta, y, rinv, sh);
+}
+
+DEV void cluster_sync() {
+  __syncthreads();  // converged warps: the barrier instructions are .aligned
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// The whole reduced solve of a column in one launch, for a general Hbar (gdr_dense_gmres_sh):
+// a cluster of ns CTAs, the base solve in the first; the others factor their own shifted
+// matrices meanwhile, meet it at the cluster barrier, then take its s through the kept
+// reflectors.  As two launches the shifts' factorisations waited for the base solve (m = 40,
+// six shifts: 500 us).
+__global__ void __launch_bounds__(DT) dense_sh_cluster_kernel(DenseCycle d) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ Sh sh;
+  c128* A = reinterpret_cast<c128*>(smem_raw);
+  const int c = blockIdx.y, i = blockIdx.x;
+  ColState* st = d.st + c;
+  if (!st->active) return;  // the whole cluster
+  if (i == 0) {
+    base_ls(d, c, A, sh);
+    cluster_sync();
+    return;
+  }
+  const int m = d.m, me = st->m_eff, rows = me + 1, lda = odd_ld(rows);
+  c128* keep = A + (long)lda * (me + 2);
+  c128* y = keep + 2 * (me + 1);
+  c128* rinv = y + (me + 1);
+  const c128* H = d.H + (long)c * (m + 1) * m;
+  const c128* cv = d.cvec + (long)c * (m + 1);
+  load_shifted(A, lda, H, m + 1, rows, me, d.sigma[(long)c * d.ns + i]);
+  for (int r = threadIdx.x; r < rows; r += DT) A[r + (long)me * lda] = cv[r];
+  __syncthreads();
+  cta_qr_r(A, lda, rows, me, me + 1, sh, d.kfull, keep);
+  cluster_sync();
+  if (!d.sact[(long)c * d.ns + i]) {  // frozen shift: no update
+    for (int r = threadIdx.x; r <= m; r += DT) d.Cf[(long)c * d.ccs + r + (long)i * d.ldc] = {0, 0};
+    return;
+  }
+  if (threadIdx.x < 32) {
+    const c128* s = d.s + (long)c * (m + 1);
+    c128 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = threadIdx.x + 32 * q;
+      v[q] = r < rows ? s[r] : c128{0, 0};
+    }
+    apply_kept(A, lda, rows, me, d.kfull, keep, v);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = threadIdx.x + 32 * q;
+      if (r < rows) A[r + (long)(me + 1) * lda] = v[q];
     }
   }
-  for (int r = threadIdx.x; r < me; r += DT)
-    y[r] = beta * A[r + (long)me * lda] - bnew * A[r + (long)(me + 1) * lda];
   __syncthreads();
-  if (!fast_backsolve(A, lda, me, y, rinv, sh)) set_err(st, GDR_EBREAKDOWN);
-  for (int r = threadIdx.x; r <= m; r += DT) Cf[r + (long)col * d.ldc] = (r < me) ? y[r] : c128{0, 0};
-  if (threadIdx.x == 0) {
-    d.beta[(long)c * d.ns + i] = bnew;
-    d.norms[(long)c * d.ns + i] = cabs_(bnew) * st->rnorm;
-  }
+  const c128 beta = d.beta[(long)c * d.ns + i];
+  shift_finish(d, c, i, A, lda, beta, y, rinv, sh);
 }
 
 // --------------------------------------------------- harmonic Ritz (D1)
@@ -1762,7 +1874,33 @@ size_t dense_smem_bytes(int m, int k) {
   return sizeof(c128) * std::max(a, std::max(b, r));
 }
 
+constexpr int DENSE_CLUSTER = 8;
+// shared memory of dense_sh_cluster_kernel: the matrix with c and s, kept scalars, y, 1/R_jj;
+// at least what base_ls uses
+static size_t cluster_smem(int m) { return sizeof(c128) * ((size_t)odd_ld(m + 1) * (m + 2) + 4 * (size_t)(m + 1) + 8); }
+
+// whether clusters of the largest size and shared memory can be resident
+static bool cluster_fits(gdr_ctx* ctx) {
+  if (set_max_dyn_smem(ctx, dense_sh_cluster_kernel) < cluster_smem(GDR_MAX_M)) return false;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim = {DENSE_CLUSTER, 1, 1};
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(DENSE_CLUSTER);
+  cfg.blockDim = dim3(DT);
+  cfg.dynamicSmemBytes = cluster_smem(GDR_MAX_M);
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, dense_sh_cluster_kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return n > 0;
+}
+
 void dense_init(gdr_ctx* ctx) {
+  ctx->dense_cluster = cluster_fits(ctx);
   size_t lim = set_max_dyn_smem(ctx, dense_d1_kernel);
   lim = std::min(lim, set_max_dyn_smem(ctx, dense_d2_kernel));
   lim = std::min(lim, set_max_dyn_smem(ctx, proj_gj_setup_kernel));
@@ -1799,6 +1937,23 @@ void dense_restart(gdr_ctx* ctx, const DenseCycle& dc) {
 void dense_cycle(gdr_ctx* ctx, const DenseCycle& dc) {
   DenseCycle d = dc;
   const size_t smem = cycle_smem(ctx, d);
+  if (d.k == 0 && !d.fom && !d.ls32 && d.kfull > d.m && d.ns >= 2 && d.ns <= DENSE_CLUSTER && ctx->dense_cluster) {
+    // a general Hbar: base solve and shifts in one cluster (at most eight CTAs, the portable size)
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim = {(unsigned)d.ns, 1, 1};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)d.ns, (unsigned)d.ncol);
+    cfg.blockDim = dim3(DT);
+    cfg.dynamicSmemBytes = cluster_smem(d.m);
+    cfg.stream = ctx->stream;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    KProf kp(ctx, "dense_sh_cluster", 0.0);
+    GDR_CUDA(cudaLaunchKernelEx(&cfg, dense_sh_cluster_kernel, d));
+    GDR_LAUNCHED(ctx);
+    return;
+  }
   dim3 g1(d.k > 0 ? 2 : 1, (unsigned)d.ncol);
   {
     KProf kp(ctx, d.k > 0 ? "dense_ls_harmonic_ritz" : "dense_ls", 0.0);

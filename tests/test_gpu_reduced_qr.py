@@ -5,7 +5,9 @@ remaining columns in one pass, up to four passes of 32 columns.  m = 1 (one refl
 8 and 14 / 15 / 16 columns (where the lane count changes with the last ones), 31 (one pass of
 32), 32, 64 and 96 (two, three, four passes).  Against numpy's FP64 solve of the same systems,
 relative to the norm of each result: 1e-13 times the condition number of the system (backward
-error of Householder QR, a modest multiple of m 2^-53)."""
+error of Householder QR, a modest multiple of m 2^-53).  Two to eight shifts are one cluster
+of as many CTAs, whose shifts apply the kept reflectors to the base solve's residual; one and
+nine shifts take the two launches."""
 import numpy as np
 import pytest
 
@@ -29,14 +31,14 @@ def ctx():
     g.gdr_destroy(c)
 
 
-@pytest.mark.parametrize("m", [1, 2, 6, 7, 8, 14, 15, 16, 31, 32, 64, 96])
-def test_reduced_solve_sizes(ctx, m):
-    ns = 3
+@pytest.mark.parametrize("m,ns", [(m, 3) for m in (1, 2, 6, 7, 8, 14, 15, 16, 31, 32, 64, 96)] +
+                         [(33, 1), (33, 2), (33, 8), (33, 9), (95, 8)])
+def test_reduced_solve_sizes(ctx, m, ns):
     r = np.random.default_rng(m)
     H = (r.standard_normal((m + 1, m)) + 1j * r.standard_normal((m + 1, m))) / np.sqrt(m)
     c = r.standard_normal(m + 1) + 1j * r.standard_normal(m + 1)
-    sig = np.array([-2.0, -2.5 + 0.5j, -4.0])
-    beta = np.array([1.0, 0.7 - 0.2j, -1.3j])
+    sig = -2.0 - 0.6 * np.arange(ns) + 0.5j * (np.arange(ns) % 2)
+    beta = np.concatenate([[1.0], r.standard_normal(ns - 1) + 1j * r.standard_normal(ns - 1)])
     D, s, bn, nrm = (torch.zeros(sh, dtype=dt, device="cuda") for sh, dt in (
         ((ns, m), torch.complex128), ((m + 1,), torch.complex128), ((ns,), torch.complex128), ((ns,), torch.float64)))
     g.gdr_dense_gmres_sh(ctx, m, sig, dev(np.ascontiguousarray(H.T)), dev(c), dev(beta), D, s, bn, nrm)
