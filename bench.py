@@ -696,7 +696,7 @@ def dense_flops(name, m, k, ns, ncol):
     return 0.0
 
 
-KERNEL_SOURCES = {"dcgs2_update_c64": "krylov.cu", "dcgs2_dot_c64": "krylov.cu",
+KERNEL_SOURCES = {"dcgs2_update_c64": "dcgs2.cu", "dcgs2_dot_c64": "dcgs2.cu",
                   "wilson_matvec_c64_bf16links": "ops.cu", "wilson_matvec_c64": "ops.cu"}
 
 

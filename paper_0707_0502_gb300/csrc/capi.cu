@@ -716,7 +716,6 @@ gdr_status gdr_arnoldi_cycle(gdr_ctx* ctx, const gdr_op* A, gdr_prec prec, void*
       b.ldv = pad_ld(n);
       b.vcs = b.ldv * (m + 1);
       b.V = ctx->get<cx<R>>("cyc.V", (size_t)b.vcs);
-      GDR_CUDA(cudaMemsetAsync(b.V, 0, sizeof(cx<R>) * b.vcs, ctx->stream));  // columns a breakdown leaves: 0
       // the given columns, in the library's vector order
       if (A->kind == OP_WILSON)
         op_order<cx<R>>(ctx, A, j0 + 1, static_cast<const cx<R>*>(V), n, b.V, b.ldv, true);
@@ -770,6 +769,14 @@ gdr_status gdr_arnoldi_cycle(gdr_ctx* ctx, const gdr_op* A, gdr_prec prec, void*
       GDR_CUDA(cudaMemcpyAsync(&out, b.st, sizeof(out), cudaMemcpyDeviceToHost, ctx->stream));
       GDR_CUDA(cudaStreamSynchronize(ctx->stream));
       if (m_eff) *m_eff = out.broke ? out.m_eff : m;
+      if (out.broke) {  // columns the breakdown left: 0 (here, not by clearing the basis before every cycle)
+        const int c0 = std::max(out.m_eff, j0 + 1);
+        if (c0 <= m) {
+          GDR_CUDA(cudaMemsetAsync(static_cast<cx<R>*>(V) + (long)c0 * n, 0, sizeof(cx<R>) * n * (m + 1 - c0),
+                                   ctx->stream));
+          GDR_CUDA(cudaStreamSynchronize(ctx->stream));
+        }
+      }
       if (out.nan) throw gdr_error(GDR_ENAN, "NaN/Inf in the Arnoldi recurrence");
       if (out.err) throw gdr_error((gdr_status)out.err, "a wait in the Arnoldi recurrence gave up");
     };
