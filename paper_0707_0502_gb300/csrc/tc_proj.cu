@@ -915,7 +915,15 @@ bool tc_restart(gdr_ctx* ctx, long n, int ncol, c64* V, long ldv, long vcs, int 
   TuArgs a{};
   const int nn = nout + nx;
   tc_combine_sizes(a, nv);
-  if (nv < 1 || nv > GDR_MAX_M + 1 || nn < 1 || nn > TU_MAXOUT || !ctx->tc_ok || !ctx->tc_update_ok ||
+  // The hand-overs per K atom cost the same however few outputs there are, the CUDA-core form's
+  // products grow with both, and its row tile of many vectors leaves fewer blocks on an SM; the
+  // vectors' length hardly moves the crossover.  us, CUDA cores -> here, at n = 3,072 / 49,152 /
+  // 786,432:
+  //   41 vectors, 20 outputs  10.8 -> 10.9 / 23.0 -> 25.1 / 233 -> 242;  26 outputs 1.06 / 1.07 / 1.13x
+  //   51 vectors, 20 outputs  0.86 / 0.93 / 0.99x;                       26 outputs 1.04 / 1.08 / 1.18x
+  //   61 vectors, 10 outputs  0.99 / 0.76 / 0.87x;                       15 outputs 1.09 / 1.09 / 1.17x
+  if (nn < (nv > 60 ? 16 : 26)) return false;
+  if (nv < 1 || nv > GDR_MAX_M + 1 || nn > TU_MAXOUT || !ctx->tc_ok || !ctx->tc_update_ok ||
       tc_combine_smem(a.ka, (nn + 15) / 16 * 16, TU_MINRAW, 1) > ctx->tc_combine_smem)
     return false;
   a.n = n;

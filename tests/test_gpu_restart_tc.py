@@ -11,9 +11,10 @@ accumulation (194 x 2^-24) stays below 2^-16, as do the coefficients' rounding t
 (2^-24), the dropped lo*lo product and the low parts' rounding (2^-21 together).  The
 median error is held to FP32's level, far from a single TF32 product's 2^-11.
 
-Sizes: row tiles of 64 (ragged ends, fewer rows than one tile), K atoms of 16 vectors (one,
-full, seven), MMA widths in steps of 16, odd n and a ragged CSR-batch-like length, and
-coefficients that do not fit (the CUDA-core form's bound is the same)."""
+Sizes: row tiles of 64 (ragged ends, fewer rows than one tile), K atoms of 16 vectors (two,
+three, six, seven), MMA widths in steps of 16, odd n, and both sides of the lines to the CUDA
+cores: fewer than 26 outputs (16 with more than 60 vectors) and coefficients that do not fit
+(the CUDA-core form's bound is the same)."""
 import numpy as np
 import pytest
 
@@ -38,9 +39,15 @@ def ctx():
 
 
 @pytest.mark.parametrize("n,nv,nout,nx", [
-    (40, 2, 1, 0),           # less than one row tile, one K atom
-    (64, 16, 16, 1),         # exactly one tile, one full K atom, N = 17
-    (3001, 17, 9, 3),        # odd n, two K atoms
+    (40, 2, 1, 0),           # few outputs: CUDA cores
+    (64, 16, 16, 1),
+    (3001, 17, 9, 3),
+    (40, 26, 26, 0),         # less than one row tile, the fewest outputs
+    (64, 32, 32, 1),         # exactly one tile, two full K atoms, N = 33
+    (3001, 33, 23, 3),       # odd n, three K atoms
+    (3001, 60, 25, 0),       # the last on the CUDA cores
+    (3001, 61, 15, 0),       # the same with more vectors
+    (3001, 61, 12, 4),       # N = 16
     (19456, 41, 21, 10),     # two tiles per CTA
     (4097, 81, 41, 0),       # six K atoms
     (100000, 61, 31, 8),     # many tiles per CTA: the ring of K atoms wraps
