@@ -93,7 +93,8 @@ __global__ void csr_kernel(long n, const int* __restrict__ rowptr, const int* __
 // holds the 256-row tiles the problems have (tiles: problem and tile), not the largest
 // problem's for all: of 64 problems with sides 32 to 256 two thirds of those were empty
 // (36.3 -> 35.0 us; requesting a row's entries together or staging them in shared memory
-// costs more occupancy than it hides: 37.6 and 46.7 us).  y: columns per problem; col_inner: they are the fastest blocks instead.
+// costs more occupancy than it hides: 37.6 and 46.7 us).  y: columns per problem; col_inner:
+// they are the fastest blocks instead.
 template <typename R, typename VT, int TPR>
 __global__ void csr_batch_kernel(const long* __restrict__ rp_off, const long* __restrict__ nz_off,
                                  const int* __restrict__ nrow, const int2* __restrict__ tiles,
