@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_proj_dot_kernel(const __grid
 // an atom into A while the MMAs of the one before run.  Any basis size streams through the same
 // shared memory (the restart's 81 vectors are six atoms).  The outputs leave by bulk stores or
 // reductions from shared memory.  Measured at 24^3x32 (5.3 M rows): 41 vectors x 120 columns
-// 4.07 -> 2.02 ms (86% of the copy bandwidth); the restart of 81 vectors to 41, before on the
+// 4.07 -> 1.97 ms (89% of the copy bandwidth); the restart of 81 vectors to 41, before on the
 // CUDA cores, 6.35 -> 3.0 ms, bound by its per-atom hand-overs (~1,650 cycles each).
 
 constexpr int TU_ROWS = 64;         // complex rows per tile: 128 real MMA rows
@@ -595,8 +595,7 @@ __global__ void __launch_bounds__(TU_THREADS, 1) tc_combine_kernel(const __grid_
     }
     for (long q = grp; q < natoms; q += TU_STAGES) {
       const int s = grp, rs = (int)(q % a.nraw), at = (int)(q % a.ka);
-      const bool ok = mbar_wait(&rfull[rs], (unsigned)((q / a.nraw) & 1), abort) &&
-                      (q < TU_STAGES || mbar_wait(&aempty[s], (unsigned)((q / TU_STAGES - 1) & 1), abort));
+      bool ok = mbar_wait(&rfull[rs], (unsigned)((q / a.nraw) & 1), abort);
       if (!__all_sync(0xffffffffu, ok)) break;
       const unsigned char* src = raw + (size_t)rs * TU_RAW + jl * TU_RAW_ROW + i0 * 8;
       unsigned char* hi = A + (size_t)s * 2 * TU_ATOM_A;
@@ -607,6 +606,11 @@ __global__ void __launch_bounds__(TU_THREADS, 1) tc_combine_kernel(const __grid_
         v[e] = make_float2(0.f, 0.f);
         if (4 * (e & 3) < jn) v[e] = *reinterpret_cast<const float2*>(src + 4 * (e & 3) * TU_RAW_ROW + 64 * (e >> 2));
       }
+      // the copies are in registers by the time the MMAs give the stage back (waited for together
+      // with the copies: 41 vectors x 120 columns at 24^3x32 2.034 ms, now 1.973; a third stage
+      // of A with a group of its own: the restart 3.01 -> 3.19 ms)
+      ok = q < TU_STAGES || mbar_wait(&aempty[s], (unsigned)((q / TU_STAGES - 1) & 1), abort);
+      if (!__all_sync(0xffffffffu, ok)) break;
 #pragma unroll
       for (int e = 0; e < TU_PER; ++e) {
         const int t = e & 3, h = e >> 2;
