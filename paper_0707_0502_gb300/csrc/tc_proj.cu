@@ -126,16 +126,20 @@ DEV void tmem_add16(uint32_t t0, uint32_t t1, float (&v)[16]) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]) + __uint_as_float(r[16 + i]);
 }
 
-DEV void tmem_ld16(uint32_t t, float (&v)[16]) {
-  uint32_t r[16];
+// v += t0 + (t1 + t2), 16 columns each, one wait for the three loads
+DEV void tmem_acc16(uint32_t t0, uint32_t t1, uint32_t t2, float (&v)[16]) {
+  uint32_t r[48];
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%48];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%49];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47}, [%50];\n\t"
       "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(t)
+      : "=&r"(r[0]), "=&r"(r[1]), "=&r"(r[2]), "=&r"(r[3]), "=&r"(r[4]), "=&r"(r[5]), "=&r"(r[6]), "=&r"(r[7]), "=&r"(r[8]), "=&r"(r[9]), "=&r"(r[10]), "=&r"(r[11]), "=&r"(r[12]), "=&r"(r[13]), "=&r"(r[14]), "=&r"(r[15]), "=&r"(r[16]), "=&r"(r[17]), "=&r"(r[18]), "=&r"(r[19]), "=&r"(r[20]), "=&r"(r[21]), "=&r"(r[22]), "=&r"(r[23]), "=&r"(r[24]), "=&r"(r[25]), "=&r"(r[26]), "=&r"(r[27]), "=&r"(r[28]), "=&r"(r[29]), "=&r"(r[30]), "=&r"(r[31]), "=&r"(r[32]), "=&r"(r[33]), "=&r"(r[34]), "=&r"(r[35]), "=&r"(r[36]), "=&r"(r[37]), "=&r"(r[38]), "=&r"(r[39]), "=&r"(r[40]), "=&r"(r[41]), "=&r"(r[42]), "=&r"(r[43]), "=&r"(r[44]), "=&r"(r[45]), "=&r"(r[46]), "=&r"(r[47])
+      : "r"(t0), "r"(t1), "r"(t2)
       : "memory");
 #pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 16; ++i)
+    v[i] += __uint_as_float(r[i]) + (__uint_as_float(r[16 + i]) + __uint_as_float(r[32 + i]));
 }
 
 // accumulator layout in tensor memory: D_re in columns [0, nt), D_im from column im_off
@@ -684,7 +688,9 @@ __global__ void __launch_bounds__(TU_THREADS, 1) tc_combine_kernel(const __grid_
         const bool got = mbar_wait(&dfull[b], (unsigned)((db >> 1) & 1), &own);
         if (!got) *abort = 1;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        ok = !named_any(1 + half, 128, !got);  // the group's four warps, which synchronise below, leave together
+        // the group's four warps, which synchronise to stage outputs, leave together: told here, or
+        // (restart, whose warps drain the atoms of a tile each at its own pace) at the tile's end
+        ok = MODE == TU_RESTART ? __all_sync(0xffffffffu, got) : !named_any(1 + half, 128, !got);
         if (!ok) break;
         const uint32_t tb = tm + lane_base + (uint32_t)(b * TU_DW);
         if (MODE == TU_RESTART) {
@@ -692,11 +698,7 @@ __global__ void __launch_bounds__(TU_THREADS, 1) tc_combine_kernel(const __grid_
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
               const uint32_t col = (uint32_t)(half * 32 + 16 * h);
-              float lo[16], hi[16];
-              tmem_add16(tb + ne + col, tb + TU_DLO + col, lo);  // the products with a lo part
-              tmem_ld16(tb + col, hi);
-#pragma unroll
-              for (int j = 0; j < 16; ++j) sum[16 * h + j] += hi[j] + lo[j];
+              if (col < (uint32_t)ne) tmem_acc16(tb + col, tb + ne + col, tb + TU_DLO + col, *reinterpret_cast<float(*)[16]>(sum + 16 * h));
             }
           }
         } else {
@@ -724,6 +726,7 @@ __global__ void __launch_bounds__(TU_THREADS, 1) tc_combine_kernel(const __grid_
         __syncwarp();
         if (lane == 0) mbar_arrive(&dempty[b]);
       }
+      if (MODE == TU_RESTART) ok = !named_any(1 + half, 128, !ok);
       if (!ok) break;
       if (MODE == TU_RESTART) {
         const bool bulk = a.bulk && (n % 2 == 0 || n - r0 >= TU_ROWS);  // not for an odd last row
