@@ -126,6 +126,12 @@ DEV void tmem_add16(uint32_t t0, uint32_t t1, float (&v)[16]) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]) + __uint_as_float(r[16 + i]);
 }
 
+// box of a 3-D map from shared memory (128-byte aligned), in the thread's bulk group
+DEV void tma_store_3d(const CUtensorMap* map, int x, int y, int z, const void* src) {
+  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(map), "r"(x),
+               "r"(y), "r"(z), "r"(s_addr(src))
+               : "memory");
+}
 // v += t0 + (t1 + t2), 16 columns each, one wait for the three loads
 DEV void tmem_acc16(uint32_t t0, uint32_t t1, uint32_t t2, float (&v)[16]) {
   uint32_t r[48];
@@ -328,7 +334,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_proj_dot_kernel(const __grid
 // shared memory (the restart's 81 vectors are six atoms).  The outputs leave by bulk stores or
 // reductions from shared memory.  Measured at 24^3x32 (5.3 M rows): 41 vectors x 120 columns
 // 4.07 -> 1.97 ms (89% of the copy bandwidth); the restart of 81 vectors to 41, before on the
-// CUDA cores, 6.35 -> 3.0 ms, bound by its per-atom hand-overs (~1,650 cycles each).
+// CUDA cores, 6.35 -> 2.43 ms, bound by its epilogue warps (a drain per atom and the outputs).
 
 constexpr int TU_ROWS = 64;         // complex rows per tile: 128 real MMA rows
 constexpr int TU_THREADS = 640;     // warp 0 copies of V, warps 1 and 3 MMA, warp 2 tensor memory, warps 4-11 A atoms, warps 12-19 epilogue
@@ -365,6 +371,7 @@ struct TuArgs {
   float* R;                  // R as floats, column k at R + 2 * k * ldr
   long ldr;
   int nout;                  // TU_RESTART: columns written into V; the others go to X
+  int tstore;                // ... whole tiles of them by tensor stores (mapO)
   c128* X;
   long ldx, xcs;
   const ColState* st;
@@ -400,7 +407,8 @@ DEV bool named_any(int id, int threads, bool p) {
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(TU_THREADS, 1) tc_combine_kernel(const __grid_constant__ CUtensorMap mapV, TuArgs a) {
+__global__ void __launch_bounds__(TU_THREADS, 1) tc_combine_kernel(const __grid_constant__ CUtensorMap mapV,
+                                                                  const __grid_constant__ CUtensorMap mapO, TuArgs a) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -647,7 +655,8 @@ __global__ void __launch_bounds__(TU_THREADS, 1) tc_combine_kernel(const __grid_
     // columns [k0, k0 + TU_SC) x 128 rows through shared memory, one 512-byte bulk store or
     // reduction per column (fewer at the ragged end): no thread waits for R's old values or
     // for its stores.  The stage's previous columns must have been read out first.
-    auto stage_out = [&](const float* d, int k0, int kend, float* out, long ld, const int* map, unsigned bytes, bool add) {
+    auto stage_out = [&](const float* d, int k0, int kend, float* out, long ld, const int* map, unsigned bytes, bool add,
+                         int tx) {
       if (a.nstage == 2) {
         stage = stage == stage0 ? stage0 + TU_SC * 128 : stage0;
         asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
@@ -659,7 +668,9 @@ __global__ void __launch_bounds__(TU_THREADS, 1) tc_combine_kernel(const __grid_
       for (int j = 0; j < TU_SC; ++j) stage[j * 128 + m] = d[j];
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       named_sync(1 + half, 128);
-      if (m < TU_SC && k0 + m < kend) {
+      if (MODE == TU_RESTART && tx >= 0) {
+        if (m == 0) tma_store_3d(&mapO, tx, k0, batch, stage);
+      } else if (m < TU_SC && k0 + m < kend) {
         float* dst = out + 2 * (long)(map ? col0 + map[k0 + m] : k0 + m) * ld;
         if (add)
           asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(
@@ -698,7 +709,8 @@ __global__ void __launch_bounds__(TU_THREADS, 1) tc_combine_kernel(const __grid_
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
               const uint32_t col = (uint32_t)(half * 32 + 16 * h);
-              if (col < (uint32_t)ne) tmem_acc16(tb + col, tb + ne + col, tb + TU_DLO + col, *reinterpret_cast<float(*)[16]>(sum + 16 * h));
+              if (col < (uint32_t)ne)  // the products with a lo part first, then the sum so far
+                tmem_acc16(tb + col, tb + ne + col, tb + TU_DLO + col, *reinterpret_cast<float(*)[16]>(sum + 16 * h));
             }
           }
         } else {
@@ -710,7 +722,7 @@ __global__ void __launch_bounds__(TU_THREADS, 1) tc_combine_kernel(const __grid_
               tmem_add16(tb + (uint32_t)k0, tb + (uint32_t)(TU_DLO + k0), d);
               if (MODE == TU_REDUCE) {
                 const unsigned bytes = (unsigned)min(128L, 2 * n - 2 * r0) * 4u;  // n even: a multiple of 16
-                stage_out(d, k0, nact, a.R + 2 * r0, a.ldr, cmap, bytes, true);
+                stage_out(d, k0, nact, a.R + 2 * r0, a.ldr, cmap, bytes, true, -1);
               } else {
 #pragma unroll
                 for (int j = 0; j < TU_SC; ++j) {
@@ -736,7 +748,10 @@ __global__ void __launch_bounds__(TU_THREADS, 1) tc_combine_kernel(const __grid_
         for (int h = 0; h < 2; ++h) {
           const int k0 = half * 32 + TU_SC * h, k1 = min(k0 + TU_SC, nact);
           if (k0 >= nact) break;  // uniform in the group
-          stage_out(sum + TU_SC * h, k0, bulk ? min(a.nout, k1) : 0, Vf, a.ldv, nullptr, bytes, false);
+          // a whole tile: one tensor store of the 16 columns (clipped at nout), where 16 bulk stores
+          // held the group up while the MMAs waited for it (81 -> 41 at 24^3x32: 2.98 ms, now 2.43)
+          const int tx = a.tstore && n - r0 >= TU_ROWS && k0 < a.nout ? (int)(2 * r0) : -1;
+          stage_out(sum + TU_SC * h, k0, bulk ? min(a.nout, k1) : 0, Vf, a.ldv, nullptr, bytes, false, tx);
           if (!rowok) continue;
           // each thread reads back its own row: a loop over just these columns (unrolled over
           // `sum` the compiler predicates all 32 FP64 additions, and the pipe runs each)
@@ -877,7 +892,9 @@ static void tc_combine_launch(gdr_ctx* ctx, TuArgs& a, unsigned gx, unsigned gy)
   CUtensorMap mv = {};
   a.bulk = a.ldv % 2 == 0 && a.vcs % 2 == 0 && (reinterpret_cast<uintptr_t>(a.V) & 15) == 0 && a.n < (1L << 29) &&
            make_map_raw(mv, a.V, a.n, a.ldv, a.nv, a.vcs, MODE == TU_RESTART ? (int)gy : 1);
-  tc_combine_kernel<MODE><<<dim3(gx, gy), TU_THREADS, tc_combine_smem(a.ka, ne, a.nraw, a.nstage), ctx->stream>>>(mv, a);
+  CUtensorMap mo = {};
+  a.tstore = MODE == TU_RESTART && a.bulk && a.nout > 0 && make_map_raw(mo, a.V, a.n, a.ldv, a.nout, a.vcs, (int)gy);
+  tc_combine_kernel<MODE><<<dim3(gx, gy), TU_THREADS, tc_combine_smem(a.ka, ne, a.nraw, a.nstage), ctx->stream>>>(mv, mo, a);
   GDR_LAUNCHED(ctx);
 }
 
@@ -925,7 +942,7 @@ bool tc_restart(gdr_ctx* ctx, long n, int ncol, c64* V, long ldv, long vcs, int 
   // The hand-overs per K atom cost the same however few outputs there are, the CUDA-core form's
   // products grow with both, and its row tile of many vectors leaves fewer blocks on an SM; the
   // vectors' length hardly moves the crossover.  us, CUDA cores -> here, at n = 3,072 / 49,152 /
-  // 786,432:
+  // 786,432 (before whole tiles left by tensor stores, which only helps this side):
   //   41 vectors, 20 outputs  10.8 -> 10.9 / 23.0 -> 25.1 / 233 -> 242;  26 outputs 1.06 / 1.07 / 1.13x
   //   51 vectors, 20 outputs  0.86 / 0.93 / 0.99x;                       26 outputs 1.04 / 1.08 / 1.18x
   //   61 vectors, 10 outputs  0.99 / 0.76 / 0.87x;                       15 outputs 1.09 / 1.09 / 1.17x
