@@ -615,8 +615,8 @@ namespace {
 // other from shared memory, six contiguous runs.  Bound by HBM; the element-wise form it
 // replaces gathered 8 or 16 bytes per thread 96 or 192 bytes apart after a 64-bit division
 // each (5.3 M x 12 complex64: 290 us, against 150 us for one read and one write).
-// Complex64 vectors that are not 16-byte aligned (pairs split across units) take the
-// element-wise form below.
+// Vectors that do not start on 16-byte boundaries (the C interface promises the alignment of
+// a real number only) take the element-wise form below, in words of 8 bytes.
 constexpr int OS = 64;
 struct SigmaArg {  // shifts passed by value on the way, stored for the kernel that follows
   int n;
@@ -652,14 +652,16 @@ __global__ void __launch_bounds__(128) wilson_order_kernel(long V, const T* __re
     for (int t = threadIdx.x; t < tot; t += 128) dst[s0 * UP + t] = buf[t];
   }
 }
-__global__ void wilson_order_elem_kernel(long V, const c64* __restrict__ in, long ldi, c64* __restrict__ out, long ldo,
-                                         int to_lib) {
+// K words of 8 bytes per component; strides in words
+template <int K>
+__global__ void wilson_order_elem_kernel(long V, const float2* __restrict__ in, long ldi, float2* __restrict__ out,
+                                         long ldo, int to_lib) {
   const int c = blockIdx.y;
-  const long n = 12 * V;
+  const long n = 12 * V * K;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const long pv = i >> 1;
+    const long pv = i / (2 * K);
     const long p = pv / V, site = pv - p * V;
-    const long u = site * 12 + 2 * p + (i & 1);
+    const long u = site * (12 * K) + 2 * K * p + i % (2 * K);
     if (to_lib) out[c * ldo + i] = in[c * ldi + u];
     else out[c * ldo + u] = in[c * ldi + i];
   }
@@ -673,15 +675,15 @@ static bool aligned16(const void* p, long ld_bytes, int cols) {
 template <typename T>
 static void wilson_order_launch(gdr_ctx* ctx, long V, int cols, const T* in, long ldi, T* out, long ldo, bool to_lib,
                                 const SigmaArg& sg, c128* sdst) {
-  if constexpr (sizeof(T) == 8) {
-    if (!aligned16(in, ldi * 8, cols) || !aligned16(out, ldo * 8, cols)) {
-      dim3 grid((unsigned)std::min<long>((12 * V + 255) / 256, 8L * ctx->num_sms), (unsigned)cols);
-      wilson_order_elem_kernel<<<grid, 256, 0, ctx->stream>>>(V, in, ldi, out, ldo, to_lib ? 1 : 0);
-      GDR_LAUNCHED(ctx);
-      if (sdst)
-        GDR_CUDA(cudaMemcpyAsync(sdst, sg.v, sizeof(c128) * sg.n, cudaMemcpyHostToDevice, ctx->stream));
-      return;
-    }
+  if (!aligned16(in, ldi * sizeof(T), cols) || !aligned16(out, ldo * sizeof(T), cols)) {
+    constexpr int K = sizeof(T) / 8;
+    dim3 grid((unsigned)std::min<long>((12 * K * V + 255) / 256, 8L * ctx->num_sms), (unsigned)cols);
+    wilson_order_elem_kernel<K><<<grid, 256, 0, ctx->stream>>>(V, reinterpret_cast<const float2*>(in), ldi * K,
+                                                               reinterpret_cast<float2*>(out), ldo * K, to_lib ? 1 : 0);
+    GDR_LAUNCHED(ctx);
+    if (sdst)
+      GDR_CUDA(cudaMemcpyAsync(sdst, sg.v, sizeof(c128) * sg.n, cudaMemcpyHostToDevice, ctx->stream));
+    return;
   }
   wilson_order_kernel<T><<<dim3((unsigned)((V + OS - 1) / OS), (unsigned)cols), 128, 0, ctx->stream>>>(
       V, in, ldi, out, ldo, to_lib ? 1 : 0, sg, sdst);

@@ -1,0 +1,105 @@
+"""Caller's arrays that start 8 bytes off a 16-byte boundary (runs on a GB300; -m gpu).
+
+The C interface passes c128 arrays as interleaved doubles and asks for no more than a double's
+alignment.  Wilson vectors are then reordered word by word: the same permutation, so every
+call gives bit by bit what it gives for the same values at an aligned address."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from tests.gpu_util import dev, small_wilson
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no GPU", allow_module_level=True)
+
+import paper_0707_0502_gb300 as g  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import __graft_entry__
+    __graft_entry__.build()
+    c = g.gdr_create(0)
+    yield c
+    g.gdr_destroy(c)
+
+
+@pytest.fixture(scope="module")
+def wilson(ctx):
+    p, A = small_wilson(dims=(3, 3, 5, 3), nshift=2, nrhs=2)
+    op = g.make_operator(ctx, p)
+    yield p, A, op
+    g.gdr_op_destroy(op)
+
+
+def _real(t):
+    return torch.view_as_real(t).reshape(-1)
+
+
+class _Off:
+    """Doubles on the device, the first one 8 bytes behind a 16-byte boundary."""
+
+    def __init__(self, values):
+        v = _real(values)
+        self.buf = torch.full((v.numel() + 2,), -7.0, dtype=torch.float64, device="cuda")
+        assert self.buf.data_ptr() % 16 == 0
+        self.buf[1:-1] = v
+        self.ptr = self.buf.data_ptr() + 8
+
+    def get(self, like):
+        assert self.buf[0] == -7.0 and self.buf[-1] == -7.0        # nothing around the array is written
+        return torch.view_as_complex(self.buf[1:-1].clone().view(-1, 2)).view(like.shape)
+
+
+@pytest.mark.parametrize("prec", [g.GDR_PREC_FP64, g.GDR_PREC_MIXED], ids=["fp64", "mixed"])
+def test_wilson_solves(ctx, wilson, prec):
+    p, A, op = wilson
+    B = dev(p.B.T)
+    X = torch.zeros((2, 2, p.n), dtype=torch.complex128, device="cuda")
+    prm = g.gdr_params_default(m=p.m, k=p.k, m_proj=p.m_proj, tol=1e-8, prec=prec)
+    sig = np.ascontiguousarray(p.sigma, complex)
+    st, rep, defl = g.gdr_solve_multishift(ctx, op, sig, B, X, prm, want_defl=True)
+    assert st == g.GDR_OK and defl
+    Bo, Xo, rp, dh = _Off(B), _Off(torch.zeros_like(X)), g.gdr_report(), ctypes.c_void_p()
+    L = g.lib()
+    st = L.gdr_solve_multishift(ctx, op, 2, sig.ctypes.data, 2, Bo.ptr, Xo.ptr, ctypes.byref(prm), ctypes.byref(dh),
+                                ctypes.byref(rp))
+    assert st == g.GDR_OK
+    assert torch.equal(Xo.get(X), X)
+    Y = torch.zeros_like(X)
+    g.gdr_solve_proj(ctx, op, defl, sig, B, Y, prm)
+    Yo = _Off(torch.zeros_like(X))
+    assert L.gdr_solve_proj(ctx, op, defl, 2, sig.ctypes.data, 2, Bo.ptr, Yo.ptr, ctypes.byref(prm),
+                            ctypes.byref(rp)) in (g.GDR_OK, g.GDR_ENOCONV)
+    assert torch.equal(Yo.get(Y), Y)
+    V = torch.zeros((p.k + 1, p.n), dtype=torch.complex128, device="cuda")
+    g.gdr_defl_export(ctx, defl, V)
+    Vo = _Off(torch.zeros_like(V))
+    assert L.gdr_defl_export(ctx, defl, Vo.ptr, None, None) == g.GDR_OK
+    assert torch.equal(Vo.get(V), V)
+    for h in (defl, dh):
+        g.gdr_defl_destroy(h)
+
+
+def test_wilson_matvec_and_cycle_fp64(ctx, wilson):
+    p, A, op = wilson
+    r = np.random.default_rng(1)
+    X = dev(r.standard_normal((3, p.n)) + 1j * r.standard_normal((3, p.n)))
+    Y = torch.zeros_like(X)
+    sig = np.ascontiguousarray([0.0, 0.5j, 1.0], complex)
+    g.gdr_op_apply(ctx, op, g.GDR_PREC_FP64, sig, X, Y)
+    Xo, Yo = _Off(X), _Off(Y * 0)
+    assert g.lib().gdr_op_apply(ctx, op, g.GDR_PREC_FP64, 3, sig.ctypes.data, Xo.ptr, Yo.ptr) == g.GDR_OK
+    assert torch.equal(Yo.get(Y), Y)
+    m = 6
+    V = torch.zeros((m + 1, p.n), dtype=torch.complex128, device="cuda")
+    V[0] = X[0] / torch.linalg.vector_norm(X[0])
+    H = torch.zeros((m, m + 1), dtype=torch.complex128, device="cuda")
+    Vo, Ho, me = _Off(V), _Off(H), ctypes.c_int()
+    g.gdr_arnoldi_cycle(ctx, op, g.GDR_PREC_FP64, V, 0, m, H)
+    assert g.lib().gdr_arnoldi_cycle(ctx, op, g.GDR_PREC_FP64, Vo.ptr, 0, m, Ho.ptr, 0, ctypes.byref(me)) == g.GDR_OK
+    assert torch.equal(Vo.get(V), V) and torch.equal(Ho.get(H), H)
