@@ -941,9 +941,14 @@ gdr_status gdr_basis_dot(gdr_ctx* ctx, gdr_prec prec, long n, int nv, const void
     GDR_REQUIRE(V && R && C, "null argument");
     GDR_CUDA(cudaSetDevice(ctx->device));
     ctx->tc_proj = !(flags & GDR_FLAG_NO_TENSOR_CORES);
+    // the sums are written as 16-byte elements: into scratch when C has a double's alignment only
+    const bool direct = (reinterpret_cast<uintptr_t>(C) & 15) == 0;
+    c128* dots = direct ? reinterpret_cast<c128*>(C) : ctx->get<c128>("bdot.h", (size_t)(nv + 2) * ncol);
     if (prec != GDR_PREC_FP64 &&
-        gs_dot_tc(ctx, n, nv, static_cast<const c64*>(V), n, ncol, static_cast<const c64*>(R), ldr,
-                  reinterpret_cast<c128*>(C), nv, nullptr, ((double)nv + ncol) * n * sizeof(c64))) {
+        gs_dot_tc(ctx, n, nv, static_cast<const c64*>(V), n, ncol, static_cast<const c64*>(R), ldr, dots, nv, nullptr,
+                  ((double)nv + ncol) * n * sizeof(c64))) {
+      if (!direct)
+        GDR_CUDA(cudaMemcpyAsync(C, dots, sizeof(c128) * nv * ncol, cudaMemcpyDeviceToDevice, ctx->stream));
       tc_check(ctx);
       return;
     }

@@ -103,3 +103,17 @@ def test_wilson_matvec_and_cycle_fp64(ctx, wilson):
     g.gdr_arnoldi_cycle(ctx, op, g.GDR_PREC_FP64, V, 0, m, H)
     assert g.lib().gdr_arnoldi_cycle(ctx, op, g.GDR_PREC_FP64, Vo.ptr, 0, m, Ho.ptr, 0, ctypes.byref(me)) == g.GDR_OK
     assert torch.equal(Vo.get(V), V) and torch.equal(Ho.get(H), H)
+
+
+@pytest.mark.parametrize("prec,ncol", [(g.GDR_PREC_MIXED, 12), (g.GDR_PREC_MIXED, 3), (g.GDR_PREC_FP64, 3)])
+def test_projection_dots(ctx, prec, ncol):
+    """C on the tensor cores (8 columns and more) and on the CUDA cores."""
+    n, nv = 300, 9
+    r = np.random.default_rng(ncol)
+    dt = torch.complex128 if prec == g.GDR_PREC_FP64 else torch.complex64
+    V, R = (dev(r.standard_normal((k, n)) + 1j * r.standard_normal((k, n)), dt) for k in (nv, ncol))
+    C = torch.zeros((ncol, nv), dtype=torch.complex128, device="cuda")
+    g.gdr_basis_dot(ctx, prec, n, nv, V, ncol, R, n, C)
+    Co = _Off(torch.zeros_like(C))
+    assert g.lib().gdr_basis_dot(ctx, prec, n, nv, V.data_ptr(), ncol, R.data_ptr(), n, Co.ptr, 0) == g.GDR_OK
+    assert torch.equal(Co.get(C), C)
