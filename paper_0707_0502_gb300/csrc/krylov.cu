@@ -925,8 +925,10 @@ void gs_dot_shared_reserve(gdr_ctx* ctx, long n, int ncol, int nv) {
 // CUDA-core kernels are memory-bound anyway)
 constexpr int TC_MIN_COLS = 8;
 
+// vectors i0 .. i0 + nv - 1 of the basis, into h_out + i0
 template <typename R, int NVM>
-static void gs_dot_shared_launch(gdr_ctx* ctx, const Batch<R>& b, int nv, const cx<R>* w, long wcs, c128* h_out) {
+static void gs_dot_shared_launch(gdr_ctx* ctx, const Batch<R>& b, int i0, int nv, const cx<R>* w, long wcs,
+                                 c128* h_out) {
   const int S = dot_shared_slots(ctx, b.n, b.ncol);
   c128* part = ctx->get<c128>("dsh.part", (size_t)S * b.ncol * nv + 64);
   const size_t smem = sizeof(cx<R>) * NVM * DS_TR + sizeof(c128) * DS_W * NVM;
@@ -934,13 +936,19 @@ static void gs_dot_shared_launch(gdr_ctx* ctx, const Batch<R>& b, int nv, const 
   {
     KProf kp(ctx, sizeof(R) == 4 ? "gs_dot_shared_c64" : "gs_dot_shared_c128",
              ((double)nv * b.n + col_len(b)) * sizeof(cx<R>) * run_share(ctx, b));
-    gs_dot_shared_kernel<R, NVM><<<grid, DS_W * 32, smem, ctx->stream>>>(b.n, b.V, b.ldv, nv, w, wcs, b.ncol, b.st,
-                                                                          part);
+    gs_dot_shared_kernel<R, NVM><<<grid, DS_W * 32, smem, ctx->stream>>>(b.n, b.V + (long)i0 * b.ldv, b.ldv, nv, w, wcs,
+                                                                          b.ncol, b.st, part);
     GDR_LAUNCHED(ctx);
   }
   const int tot = b.ncol * nv;
-  gs_dot_shared_sum_kernel<<<(tot + 31) / 32, 256, 0, ctx->stream>>>(S, b.ncol, nv, part, h_out, b.m + 2, b.st);
+  gs_dot_shared_sum_kernel<<<(tot + 31) / 32, 256, 0, ctx->stream>>>(S, b.ncol, nv, part, h_out + i0, b.m + 2, b.st);
   GDR_LAUNCHED(ctx);
+}
+
+// whether every vector starts on a 16-byte boundary, as the kernels that load 16-byte units need
+template <typename R>
+static bool in_units(const cx<R>* p, long ld, int cols) {
+  return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (cols == 1 || ld * sizeof(cx<R>) % 16 == 0);
 }
 
 bool gs_dot_tc(gdr_ctx* ctx, long n, int nv, const c64* V, long ldv, int ncol, const c64* R, long ldr, c128* out,
@@ -964,11 +972,18 @@ void gs_dot(gdr_ctx* ctx, const Batch<R>& b, int nv, const cx<R>* w, long wcs, c
       if (gs_dot_tc(ctx, b.n, nv, b.V, b.ldv, b.ncol, w, wcs, h_out, b.m + 2, b.st, bytes)) return;
     }
   }
-  if (dot_shared_applies(b, nv, wnorm, wprev)) {  // one basis for many columns: read it once
-    if (nv <= 24) gs_dot_shared_launch<R, 24>(ctx, b, nv, w, wcs, h_out);
-    else gs_dot_shared_launch<R, 48>(ctx, b, nv, w, wcs, h_out);
+  // one basis for many columns: read it once; and what the unit kernel below cannot load (the
+  // caller's complex64 vectors at odd strides or 8-byte starts), 48 vectors at a time
+  const bool units = in_units<R>(b.V, b.ldv, nv) && in_units<R>(w, wcs, b.ncol);
+  if (dot_shared_applies(b, nv, wnorm, wprev) || (!units && b.vcs == 0 && !b.nvec && !wnorm && !wprev)) {
+    for (int i0 = 0; i0 < nv; i0 += 48) {
+      const int ni = std::min(48, nv - i0);
+      if (ni <= 24) gs_dot_shared_launch<R, 24>(ctx, b, i0, ni, w, wcs, h_out);
+      else gs_dot_shared_launch<R, 48>(ctx, b, i0, ni, w, wcs, h_out);
+    }
     return;
   }
+  GDR_REQUIRE(units, "Gram-Schmidt dot: vectors must start on 16-byte boundaries");
   int S, G;
   dot_grid(ctx, b, nv + (wnorm ? 1 : 0), S, G);
   dim3 grid((unsigned)(S * G), (unsigned)b.ncol);

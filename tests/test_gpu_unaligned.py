@@ -117,3 +117,33 @@ def test_projection_dots(ctx, prec, ncol):
     Co = _Off(torch.zeros_like(C))
     assert g.lib().gdr_basis_dot(ctx, prec, n, nv, V.data_ptr(), ncol, R.data_ptr(), n, Co.ptr, 0) == g.GDR_OK
     assert torch.equal(Co.get(C), C)
+
+
+@pytest.mark.parametrize("n,nv,ncol,pad,offv,offr", [
+    (3001, 21, 1, 0, 0, 0),       # odd n: every second vector of V starts off a boundary
+    (3001, 60, 40, 0, 0, 0),      # more vectors than one pass of the element-wise form takes
+    (3001, 97, 1, 0, 0, 0),
+    (300, 60, 3, 1, 0, 0),        # odd column stride of R
+    (300, 60, 2, 0, 1, 0),        # V, R starting 8 bytes off
+    (300, 7, 1, 0, 0, 1),
+    (300, 60, 12, 0, 1, 1),
+    (1, 2, 1, 0, 0, 0),
+])
+def test_projection_dots_of_unaligned_vectors(ctx, n, nv, ncol, pad, offv, offr):
+    """Element by element |dot - exact| <= 2^-16 S, S = sum |v||r| over the real products: a thread
+    adds at most 64 complex products in FP32 (three roundings each) before FP64 takes over."""
+    r = np.random.default_rng(n + nv)
+    V, R = ((r.standard_normal((k, n)) + 1j * r.standard_normal((k, n))).astype(np.complex64) for k in (nv, ncol))
+    Vb = torch.zeros(nv * n + 1, dtype=torch.complex64, device="cuda")
+    Rb = torch.full(((n + pad) * ncol + 1,), float("nan"), dtype=torch.complex64, device="cuda")
+    Vd = Vb[offv: offv + nv * n]
+    Rd = Rb[offr: offr + (n + pad) * ncol]
+    Vd.copy_(dev(V).view(-1))
+    Rd.view(ncol, n + pad)[:, :n] = dev(R)
+    C = torch.zeros((ncol, nv), dtype=torch.complex128, device="cuda")
+    g.gdr_basis_dot(ctx, g.GDR_PREC_MIXED, n, nv, Vd, ncol, Rd, n + pad, C, g.GDR_FLAG_NO_TENSOR_CORES)
+    got = C.cpu().numpy()
+    Vx, Rx = V.astype(complex), R.astype(complex)
+    exact = Rx @ Vx.conj().T
+    S = (np.abs(Rx.real) + np.abs(Rx.imag)) @ (np.abs(Vx.real) + np.abs(Vx.imag)).T
+    assert (np.abs(got - exact) <= 2.0 ** -16 * S).all()
