@@ -11,6 +11,13 @@
  * Conventions for every entry point
  *  - Complex numbers are interleaved (re, im) doubles: a "c128 array of length L"
  *    is 2*L doubles.  Matrices are column-major.
+ *  - Arrays start on a boundary of one element: 16 bytes for c128, 8 for complex64
+ *    (GDR_EINVAL otherwise, before any work).  A real number's alignment is enough
+ *    for B and X of the solves, for the vectors of a Wilson operator in FP64, and for
+ *    what is only copied: the arrays of a CSR operator, C of gdr_basis_dot, Hbar, c,
+ *    beta and D of gdr_dense_gmres_sh, Hbar of gdr_arnoldi_cycle, hcol, y.
+ *    gdr_arnoldi_step on a CSR operator works in the caller's V in units of 16 bytes
+ *    and wants that boundary in either precision.
  *  - Pointers are DEVICE pointers on the context's device unless the entry point
  *    says "host".  The caller owns every buffer it passes; the library owns its
  *    workspace (allocated on first use, grown on demand, freed by gdr_destroy).

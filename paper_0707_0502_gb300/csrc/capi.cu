@@ -207,6 +207,7 @@ gdr_status gdr_op_wilson(gdr_ctx* ctx, const int dims[4], double diag_a, const d
   gdr_status st = guarded(ctx, [&] {
     for (int i = 0; i < 4; ++i) GDR_REQUIRE(dims[i] >= 2, "each lattice extent must be >= 2");
     GDR_REQUIRE(links != nullptr, "null links");
+    GDR_REQUIRE_ALIGNED(links, sizeof(c128));
     GDR_REQUIRE(store == GDR_LINK_C128 || store == GDR_LINK_C64 || store == GDR_LINK_BF16, "bad link format");
     GDR_CUDA(cudaSetDevice(ctx->device));
     op->ctx = ctx;
@@ -272,6 +273,10 @@ gdr_status gdr_op_apply(gdr_ctx* ctx, const gdr_op* A, gdr_prec prec, int ncol, 
   return guarded(ctx, [&] {
     GDR_REQUIRE(ncol >= 0 && (ncol == 0 || (sigma && X && Y)), "bad gdr_op_apply arguments");
     if (ncol == 0) return;
+    // a Wilson operator's vectors are reordered, FP64 ones word by word where they must be
+    const size_t el = prec == GDR_PREC_FP64 && A->kind != OP_WILSON ? sizeof(c128) : sizeof(c64);
+    GDR_REQUIRE_ALIGNED(X, el);
+    GDR_REQUIRE_ALIGNED(Y, el);
     if (prec == GDR_PREC_FP64)
       op_apply_user<double>(ctx, A, ncol, sigma, static_cast<const c128*>(X), static_cast<c128*>(Y));
     else
@@ -646,6 +651,7 @@ gdr_status gdr_arnoldi_step(gdr_ctx* ctx, const gdr_op* A, gdr_prec prec, void* 
     GDR_REQUIRE(j >= 0 && j + 1 <= GDR_MAX_M, "j out of range");
     const long n = A->n;
     GDR_REQUIRE(prec == GDR_PREC_FP64 || n % 2 == 0, "complex64 step-level calls need an even n");
+    GDR_REQUIRE_ALIGNED(V, A->kind == OP_WILSON ? sizeof(c64) : (size_t)16);  // used in place, in 16-byte units
     auto run = [&](auto tag) {
       using R = decltype(tag);
       Batch<R> b;
@@ -704,6 +710,7 @@ gdr_status gdr_arnoldi_cycle(gdr_ctx* ctx, const gdr_op* A, gdr_prec prec, void*
   if (!ctx || !A || !V || !Hbar) return GDR_EINVAL;
   return guarded(ctx, [&] {
     GDR_REQUIRE(m >= 1 && m <= GDR_MAX_M && j0 >= 0 && j0 < m, "bad j0 / m");
+    GDR_REQUIRE_ALIGNED(V, A->kind == OP_WILSON ? sizeof(c64) : sizeof(float));
     const long n = A->n;
     GDR_REQUIRE(prec == GDR_PREC_FP64 || n % 2 == 0, "complex64 step-level calls need an even n");
     auto run = [&](auto tag) {
@@ -793,6 +800,8 @@ gdr_status gdr_dense_gmres_sh(gdr_ctx* ctx, int m, int ns, const double* Hbar, c
   return guarded(ctx, [&] {
     GDR_REQUIRE(m >= 1 && m <= GDR_MAX_M && ns >= 1, "bad sizes");
     GDR_REQUIRE(Hbar && c && sigma && beta && D && s && beta_new && norms, "null argument");
+    GDR_REQUIRE_ALIGNED(s, sizeof(c128));
+    GDR_REQUIRE_ALIGNED(beta_new, sizeof(c128));
     DenseCycle d{};
     d.ncol = 1; d.m = m; d.k = 0; d.ns = ns; d.kfull = m + 1;  // general Hbar
     c128* H = ctx->get<c128>("dstep.H", (size_t)(m + 1) * m);
@@ -835,6 +844,9 @@ gdr_status gdr_dense_ls(gdr_ctx* ctx, gdr_prec prec, int m, const double* sigma1
     GDR_REQUIRE(m >= 1 && m <= GDR_MAX_M, "bad sizes");
     GDR_REQUIRE(prec == GDR_PREC_FP64 || prec == GDR_PREC_MIXED, "prec must be GDR_PREC_FP64 or GDR_PREC_MIXED");
     GDR_REQUIRE(sigma1 && Hbar && c && y && s, "null argument");
+    GDR_REQUIRE_ALIGNED(Hbar, sizeof(c128));
+    GDR_REQUIRE_ALIGNED(c, sizeof(c128));
+    GDR_REQUIRE_ALIGNED(s, sizeof(c128));
     DenseCycle d{};
     d.ncol = 1; d.m = m; d.k = 0; d.ns = 1; d.kfull = 0;  // Hessenberg recurrence
     d.ls32 = (prec == GDR_PREC_MIXED) ? 1 : 0;
@@ -876,6 +888,12 @@ gdr_status gdr_dense_restart(gdr_ctx* ctx, gdr_prec prec, int m, int k, const do
     GDR_REQUIRE(m >= 2 && m <= GDR_MAX_M && k >= 1 && k < m, "bad sizes");
     GDR_REQUIRE(prec == GDR_PREC_FP64 || prec == GDR_PREC_MIXED, "prec must be GDR_PREC_FP64 or GDR_PREC_MIXED");
     GDR_REQUIRE(sigma1 && Hbar && s && theta && P && Hk && ck, "null argument");
+    GDR_REQUIRE_ALIGNED(Hbar, sizeof(c128));
+    GDR_REQUIRE_ALIGNED(s, sizeof(c128));
+    GDR_REQUIRE_ALIGNED(theta, sizeof(c128));
+    GDR_REQUIRE_ALIGNED(P, sizeof(c128));
+    GDR_REQUIRE_ALIGNED(Hk, sizeof(c128));
+    GDR_REQUIRE_ALIGNED(ck, sizeof(c128));
     DenseCycle d{};
     d.ncol = 1; d.m = m; d.k = k; d.ns = 1; d.kfull = m + 1;  // general Hbar
     d.hr32 = (prec == GDR_PREC_MIXED) ? 1 : 0;
@@ -924,6 +942,9 @@ gdr_status gdr_basis_update(gdr_ctx* ctx, gdr_prec prec, long n, int nv, void* V
     GDR_REQUIRE(n > 0 && nv >= 1 && nout >= 0 && nout <= nv && nx >= 0, "bad sizes");
     ctx->tc_proj = true;
     GDR_REQUIRE(V && C && (nx == 0 || X), "null argument");
+    GDR_REQUIRE_ALIGNED(V, prec == GDR_PREC_FP64 ? sizeof(c128) : sizeof(c64));
+    GDR_REQUIRE_ALIGNED(C, sizeof(c128));
+    if (nx > 0) GDR_REQUIRE_ALIGNED(X, sizeof(c128));
     if (prec == GDR_PREC_FP64)
       combine<double>(ctx, n, 1, static_cast<c128*>(V), n, 0, nv, reinterpret_cast<const c128*>(C), nv, 0, nout, nx,
                       0, reinterpret_cast<c128*>(X), n, 0, nullptr, 0, nullptr);
@@ -939,6 +960,8 @@ gdr_status gdr_basis_dot(gdr_ctx* ctx, gdr_prec prec, long n, int nv, const void
   return guarded(ctx, [&] {
     GDR_REQUIRE(n > 0 && nv >= 1 && nv <= GDR_MAX_M + 1 && ncol >= 1 && ldr >= n, "bad sizes");
     GDR_REQUIRE(V && R && C, "null argument");
+    GDR_REQUIRE_ALIGNED(V, prec == GDR_PREC_FP64 ? sizeof(c128) : sizeof(c64));
+    GDR_REQUIRE_ALIGNED(R, prec == GDR_PREC_FP64 ? sizeof(c128) : sizeof(c64));
     GDR_CUDA(cudaSetDevice(ctx->device));
     ctx->tc_proj = !(flags & GDR_FLAG_NO_TENSOR_CORES);
     // the sums are written as 16-byte elements: into scratch when C has a double's alignment only
@@ -996,6 +1019,9 @@ gdr_status gdr_basis_residual_update(gdr_ctx* ctx, gdr_prec prec, long n, int nv
   return guarded(ctx, [&] {
     GDR_REQUIRE(n > 0 && nv >= 1 && nv <= GDR_MAX_M + 1 && ncol >= 1 && ldr >= n, "bad sizes");
     GDR_REQUIRE(V && T && R, "null argument");
+    GDR_REQUIRE_ALIGNED(V, prec == GDR_PREC_FP64 ? sizeof(c128) : sizeof(c64));
+    GDR_REQUIRE_ALIGNED(T, sizeof(c128));
+    GDR_REQUIRE_ALIGNED(R, prec == GDR_PREC_FP64 ? sizeof(c128) : sizeof(c64));
     GDR_CUDA(cudaSetDevice(ctx->device));
     ctx->tc_proj = !(flags & GDR_FLAG_NO_TENSOR_CORES);
     const ColState* st = nullptr;  // every column

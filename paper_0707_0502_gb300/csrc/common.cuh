@@ -106,6 +106,11 @@ struct gdr_error : std::runtime_error {
     if (!(cond)) throw gdr_error(GDR_EINVAL, std::string(msg));                  \
   } while (0)
 
+// a caller's array that kernels access in elements of `bytes` (a null pointer passes)
+#define GDR_REQUIRE_ALIGNED(p, bytes)                                                              \
+  GDR_REQUIRE((reinterpret_cast<uintptr_t>(p) & ((bytes) - 1)) == 0,                               \
+              #p " must start on a boundary of " + std::to_string(bytes) + " bytes")
+
 // after every kernel launch
 #define GDR_LAUNCHED(ctx)                                                         \
   do {                                                                            \

@@ -86,6 +86,8 @@ extern "C" gdr_status gdr_dense_gmres_sh_noalloc(gdr_ctx* ctx, int m, int ns, co
     GDR_REQUIRE(m >= 1 && m <= NA_MAX_M, "gdr_dense_gmres_sh_noalloc: m must be in [1, GDR_NOALLOC_MAX_M]");
     GDR_REQUIRE(ns >= 1 && ns <= NA_MAX_NS, "gdr_dense_gmres_sh_noalloc: ns must be in [1, GDR_NOALLOC_MAX_NS]");
     GDR_REQUIRE(Hbar && c && sigma && beta && D && s && beta_new && norms, "null argument");
+    GDR_REQUIRE_ALIGNED(s, sizeof(c128));
+    GDR_REQUIRE_ALIGNED(beta_new, sizeof(c128));
     GDR_CUDA(cudaSetDevice(ctx->device));
     c128* base = static_cast<c128*>(scratch_address(ctx->device));
     c128* H = base;

@@ -147,3 +147,45 @@ def test_projection_dots_of_unaligned_vectors(ctx, n, nv, ncol, pad, offv, offr)
     exact = Rx @ Vx.conj().T
     S = (np.abs(Rx.real) + np.abs(Rx.imag)) @ (np.abs(Vx.real) + np.abs(Vx.imag)).T
     assert (np.abs(got - exact) <= 2.0 ** -16 * S).all()
+
+
+def test_unaligned_elements_are_refused(ctx, wilson):
+    """Arrays that kernels read element by element: GDR_EINVAL before any work, each in turn."""
+    _, _, wop = wilson
+    L, n, m, k = g.lib(), 12, 4, 2
+    op = g.gdr_op_csr(ctx, dev(np.arange(n + 1, dtype=np.int32)), dev(np.arange(n, dtype=np.int32)),
+                      dev(np.ones(n, complex)))
+    buf = torch.zeros(4000, dtype=torch.float64, device="cuda")
+    sig = np.zeros(8, complex)
+    F64, C64 = g.GDR_PREC_FP64, g.GDR_PREC_MIXED
+    A = buf.data_ptr()
+    # (call with the pointers p[0], p[1], ...; per pointer how far off it may not be, in bytes)
+    calls = [
+        (lambda p: L.gdr_op_apply(ctx, op, F64, 1, sig.ctypes.data, p[0], p[1]), [8, 8]),
+        (lambda p: L.gdr_op_apply(ctx, op, C64, 1, sig.ctypes.data, p[0], p[1]), [4, 4]),
+        (lambda p: L.gdr_op_apply(ctx, wop, C64, 1, sig.ctypes.data, p[0], p[1]), [4, 4]),
+        (lambda p: L.gdr_arnoldi_step(ctx, op, F64, p[0], 0, A), [8]),
+        (lambda p: L.gdr_arnoldi_step(ctx, op, C64, p[0], 0, A), [8]),
+        (lambda p: L.gdr_arnoldi_cycle(ctx, wop, C64, p[0], 0, 1, A, 0, None), [4]),
+        (lambda p: L.gdr_dense_gmres_sh(ctx, m, 1, A, A, sig.ctypes.data, A, A, p[0], p[1], A), [8, 8]),
+        (lambda p: L.gdr_dense_gmres_sh_noalloc(ctx, m, 1, A, A, sig.ctypes.data, A, A, p[0], p[1], A), [8, 8]),
+        (lambda p: L.gdr_dense_ls(ctx, F64, m, sig.ctypes.data, p[0], p[1], A, p[2]), [8] * 3),
+        (lambda p: L.gdr_dense_restart(ctx, F64, m, k, sig.ctypes.data, *p), [8] * 6),
+        (lambda p: L.gdr_basis_update(ctx, F64, n, 2, p[0], p[1], 1, 1, p[2]), [8] * 3),
+        (lambda p: L.gdr_basis_update(ctx, C64, n, 2, p[0], p[1], 1, 1, p[2]), [4, 8, 8]),
+        (lambda p: L.gdr_basis_dot(ctx, F64, n, 2, p[0], 1, p[1], n, A, 0), [8, 8]),
+        (lambda p: L.gdr_basis_dot(ctx, C64, n, 2, p[0], 1, p[1], n, A, 0), [4, 4]),
+        (lambda p: L.gdr_basis_residual_update(ctx, F64, n, 2, p[0], 1, p[1], p[2], n, 0), [8] * 3),
+        (lambda p: L.gdr_basis_residual_update(ctx, C64, n, 2, p[0], 1, p[1], p[2], n, 0), [4, 8, 4]),
+    ]
+    for i, (call, offs) in enumerate(calls):
+        for q, off in enumerate(offs):
+            p = [A] * len(offs)
+            p[q] += off
+            assert call(p) == g.GDR_EINVAL, (i, q)
+    import ctypes as ct
+    h, dims = ct.c_void_p(), (ct.c_int * 4)(2, 2, 2, 2)
+    assert L.gdr_op_wilson(ctx, dims, 0.0, A + 8, g.GDR_LINK_C64, ct.byref(h)) == g.GDR_EINVAL and not h.value
+    torch.cuda.synchronize()
+    assert not buf.any()
+    g.gdr_op_destroy(op)
