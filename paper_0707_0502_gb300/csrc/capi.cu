@@ -273,6 +273,7 @@ gdr_status gdr_op_apply(gdr_ctx* ctx, const gdr_op* A, gdr_prec prec, int ncol, 
   return guarded(ctx, [&] {
     GDR_REQUIRE(ncol >= 0 && (ncol == 0 || (sigma && X && Y)), "bad gdr_op_apply arguments");
     if (ncol == 0) return;
+    GDR_REQUIRE(A->kind != OP_CSR_BATCH || ncol <= A->nprob, "a CSR batch has one column per problem");
     // a Wilson operator's vectors are reordered, FP64 ones word by word where they must be
     const size_t el = prec == GDR_PREC_FP64 && A->kind != OP_WILSON ? sizeof(c128) : sizeof(c64);
     GDR_REQUIRE_ALIGNED(X, el);
