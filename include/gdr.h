@@ -24,6 +24,11 @@
  *  - Work is queued on the context's stream.  Solves synchronise that stream
  *    before returning (they read convergence words between cycles); the
  *    step-level entry points do not.
+ *  - gdr_basis_update neither waits nor checks.  Should a tensor-core wait in it give
+ *    up, the next call on the context that synchronises (operators are created all
+ *    the same) returns GDR_ETIMEOUT, whatever that call does: the update's V and X
+ *    are then unspecified, the other call's own results complete unless it ran on
+ *    the tensor cores itself.
  *  - Every entry point returns a gdr_status; on error gdr_last_error() holds a
  *    one-line message.  No C++ exception crosses the ABI.  The library never
  *    falls back to host computation: without a usable CUDA device gdr_create
@@ -317,6 +322,12 @@ gdr_status gdr_profile(gdr_ctx *ctx, int enable);
  * kernel then returns normally and the call reports GDR_ETIMEOUT, leaving the
  * context usable.  Synchronises the context stream. */
 gdr_status gdr_barrier_selftest(gdr_ctx *ctx, int rounds, int phantom);
+
+/* The same for the waits of the tensor-core kernels: queues a kernel whose one wait
+ * is for an arrival that never comes.  It gives up after about a second and leaves
+ * the mark that a gdr_basis_update leaves then, so the next call that synchronises
+ * returns GDR_ETIMEOUT and the context stays usable.  Asynchronous. */
+gdr_status gdr_tc_wait_selftest(gdr_ctx *ctx);
 gdr_status gdr_profile_report(gdr_ctx *ctx, char *buf, long len);
 
 /* --------------------------------------------------------- step-level calls
@@ -408,8 +419,9 @@ gdr_status gdr_dense_restart(gdr_ctx *ctx, gdr_prec prec, int m, int k, const do
  * X[:, i] += V C[:, nout + i] for i < nx (X c128 n x nx).
  * MIXED with 0 < nout and 26 <= nout + nx <= 64 (from 16 on with more than 60 vectors) runs on
  * the tensor cores (both factors split into two TF32 parts, FP32 accumulation: FP32
- * arithmetic's accuracy), below that on the CUDA cores in FP32.  A tensor-core wait that
- * gave up is reported by the next call that synchronises (GDR_ETIMEOUT). */
+ * arithmetic's accuracy), below that on the CUDA cores in FP32; the call has no switch.
+ * A tensor-core wait that gave up is reported by the next call that synchronises
+ * (GDR_ETIMEOUT, V and X then unspecified). */
 gdr_status gdr_basis_update(gdr_ctx *ctx, gdr_prec prec, long n, int nv, void *V, const double *C, int nout,
                             int nx, double *X);
 

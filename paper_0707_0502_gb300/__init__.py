@@ -119,6 +119,7 @@ _SIGS = {
     "gdr_dense_gmres_sh_noalloc": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_int, _P, _P, _P, _P, _P, _P, _P,
                                                   _P]),
     "gdr_barrier_selftest": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_int]),
+    "gdr_tc_wait_selftest": (ctypes.c_int, [_P]),
     "gdr_dense_ls": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_int, _P, _P, _P, _P, _P]),
     "gdr_dense_restart": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_int, ctypes.c_int, _P, _P, _P, _P, _P, _P, _P]),
     "gdr_basis_update": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_long, ctypes.c_int, _P, _P, ctypes.c_int,
@@ -400,6 +401,11 @@ def gdr_barrier_selftest(ctx, rounds, phantom):
     """Status of the grid-barrier self-test (GDR_OK, or GDR_ETIMEOUT with phantom);
     does not raise for GDR_ETIMEOUT."""
     return lib().gdr_barrier_selftest(ctx, int(rounds), int(phantom))
+
+
+def gdr_tc_wait_selftest(ctx):
+    """Queue a tensor-core wait that gives up; the next call that synchronises raises GDR_ETIMEOUT."""
+    _check(lib().gdr_tc_wait_selftest(ctx), ctx)
 
 
 def gdr_basis_update(ctx, prec, n, nv, V, C, nout, nx, X):

@@ -29,22 +29,6 @@ gdr_status guarded(gdr_ctx* ctx, F&& f) {
   }
 }
 
-// a tensor-core wait that gave up during the call (the kernel then returned without
-// its result): report it as GDR_ETIMEOUT and clear the flag for the next call
-// (waits for the stream: the flag comes behind the call's kernels, through pinned memory)
-void tc_check(gdr_ctx* ctx) {
-  int* e = static_cast<int*>(ctx->host_status(sizeof(int)));
-  *e = 0;
-  if (ctx->tc_err)
-    GDR_CUDA(cudaMemcpyAsync(e, ctx->tc_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-  GDR_CUDA(cudaStreamSynchronize(ctx->stream));
-  if (*e) {
-    GDR_CUDA(cudaMemsetAsync(ctx->tc_err, 0, sizeof(int), ctx->stream));
-    GDR_CUDA(cudaStreamSynchronize(ctx->stream));
-    throw gdr_error(GDR_ETIMEOUT, "tensor-core projection: a wait gave up");
-  }
-}
-
 void check_params(gdr_ctx* ctx, const gdr_params& p) {
   ctx->tc_proj = !(p.flags & GDR_FLAG_NO_TENSOR_CORES);
   GDR_REQUIRE(p.m >= 2 && p.m <= GDR_MAX_M, "m must be in [2, GDR_MAX_M]");
@@ -154,6 +138,7 @@ gdr_status gdr_create(gdr_ctx** out, int device, void* cuda_stream) {
     dcgs2_init(ctx);
     sweep_init(ctx);
     tc_proj_init(ctx);
+    ctx->host_status(4096);  // now, so that the step-level calls allocate nothing to report a status
   });
   if (st != GDR_OK) {
     delete ctx;
@@ -347,6 +332,7 @@ gdr_status gdr_autotune(gdr_ctx* ctx, gdr_op* A, gdr_prec prec, int ncol, int m,
     gdr_tune_result r{};
     tune_op(ctx, A, prec, ncol, m, r);
     if (out) *out = r;
+    tc_check(ctx);
   });
 }
 
@@ -588,6 +574,7 @@ gdr_status gdr_profile(gdr_ctx* ctx, int enable) {
     ctx->prof_pending.clear();
     ctx->prof.clear();
     ctx->profile = enable != 0;
+    tc_check(ctx);
   });
 }
 
@@ -618,6 +605,7 @@ gdr_status gdr_profile_report(gdr_ctx* ctx, char* buf, long len) {
     s += "}";
     GDR_REQUIRE((long)s.size() < len, "profile report buffer too small");
     std::memcpy(buf, s.c_str(), s.size() + 1);
+    tc_check(ctx);
   });
 }
 
@@ -632,7 +620,7 @@ gdr_status gdr_defl_export(gdr_ctx* ctx, const gdr_defl* defl, double* V, double
       GDR_CUDA(cudaMemcpy2DAsync(V, defl->n * sizeof(c128), defl->V128, defl->ldv * sizeof(c128),
                                  defl->n * sizeof(c128), defl->k + 1, cudaMemcpyDeviceToDevice, ctx->stream));
     if (Hbar) std::memcpy(Hbar, defl->Hk_host.data(), sizeof(c128) * defl->Hk_host.size());
-    GDR_CUDA(cudaStreamSynchronize(ctx->stream));
+    tc_check(ctx);
   });
 }
 
@@ -692,7 +680,7 @@ gdr_status gdr_arnoldi_step(gdr_ctx* ctx, const gdr_op* A, gdr_prec prec, void* 
       s.m_eff = j + 1;
       GDR_CUDA(cudaMemsetAsync(b.cnt, 0, 4 * sizeof(unsigned), ctx->stream));
       GDR_CUDA(cudaMemcpyAsync(b.st, &s, sizeof(s), cudaMemcpyHostToDevice, ctx->stream));
-      GDR_CUDA(cudaStreamSynchronize(ctx->stream));
+      tc_check(ctx);
       cx<R>* wl = nullptr;
       arnoldi_step<R>(ctx, A, b, j, j, j, wl);
       if (Vl != Vu) op_order<cx<R>>(ctx, A, 1, Vl + (long)(j + 1) * n, n, Vu + (long)(j + 1) * n, n, false);
@@ -773,9 +761,8 @@ gdr_status gdr_arnoldi_cycle(gdr_ctx* ctx, const gdr_op* A, gdr_prec prec, void*
                                    cudaMemcpyDeviceToDevice, ctx->stream));
       GDR_CUDA(cudaMemcpyAsync(Hbar + 2 * (long)(m + 1) * j0, b.H + (long)(m + 1) * j0,
                                sizeof(c128) * (m + 1) * (m - j0), cudaMemcpyDeviceToDevice, ctx->stream));
-      ColState out;
-      GDR_CUDA(cudaMemcpyAsync(&out, b.st, sizeof(out), cudaMemcpyDeviceToHost, ctx->stream));
-      GDR_CUDA(cudaStreamSynchronize(ctx->stream));
+      bool tc_failed;
+      const ColState out = fetch_state(ctx, b.st, tc_failed);
       if (m_eff) *m_eff = out.broke ? out.m_eff : m;
       if (out.broke) {  // columns the breakdown left: 0 (here, not by clearing the basis before every cycle)
         const int c0 = std::max(out.m_eff, j0 + 1);
@@ -787,6 +774,7 @@ gdr_status gdr_arnoldi_cycle(gdr_ctx* ctx, const gdr_op* A, gdr_prec prec, void*
       }
       if (out.nan) throw gdr_error(GDR_ENAN, "NaN/Inf in the Arnoldi recurrence");
       if (out.err) throw gdr_error((gdr_status)out.err, "a wait in the Arnoldi recurrence gave up");
+      if (tc_failed) tc_fail(ctx);
     };
     if (prec == GDR_PREC_FP64)
       run(double{});
@@ -831,10 +819,10 @@ gdr_status gdr_dense_gmres_sh(gdr_ctx* ctx, int m, int ns, const double* Hbar, c
     dense_cycle(ctx, d);
     GDR_CUDA(cudaMemcpy2DAsync(D, m * sizeof(c128), d.Cf, (m + 1) * sizeof(c128), m * sizeof(c128), ns,
                                cudaMemcpyDeviceToDevice, ctx->stream));
-    ColState out;
-    GDR_CUDA(cudaMemcpyAsync(&out, d.st, sizeof(out), cudaMemcpyDeviceToHost, ctx->stream));
-    GDR_CUDA(cudaStreamSynchronize(ctx->stream));
+    bool tc_failed;
+    const ColState out = fetch_state(ctx, d.st, tc_failed);
     if (out.err) throw gdr_error((gdr_status)out.err, "singular reduced system");
+    if (tc_failed) tc_fail(ctx);
   });
 }
 
@@ -875,10 +863,10 @@ gdr_status gdr_dense_ls(gdr_ctx* ctx, gdr_prec prec, int m, const double* sigma1
     GDR_CUDA(cudaStreamSynchronize(ctx->stream));
     dense_cycle(ctx, d);
     GDR_CUDA(cudaMemcpyAsync(y, d.Cf, m * sizeof(c128), cudaMemcpyDeviceToDevice, ctx->stream));
-    ColState out;
-    GDR_CUDA(cudaMemcpyAsync(&out, d.st, sizeof(out), cudaMemcpyDeviceToHost, ctx->stream));
-    GDR_CUDA(cudaStreamSynchronize(ctx->stream));
+    bool tc_failed;
+    const ColState out = fetch_state(ctx, d.st, tc_failed);
     if (out.err) throw gdr_error((gdr_status)out.err, "singular reduced system");
+    if (tc_failed) tc_fail(ctx);
   });
 }
 
@@ -918,10 +906,10 @@ gdr_status gdr_dense_restart(gdr_ctx* ctx, gdr_prec prec, int m, int k, const do
     st.m_eff = m;
     GDR_CUDA(cudaMemcpyAsync(d.st, &st, sizeof(st), cudaMemcpyHostToDevice, ctx->stream));
     dense_restart(ctx, d);
-    ColState out;
-    GDR_CUDA(cudaMemcpyAsync(&out, d.st, sizeof(out), cudaMemcpyDeviceToHost, ctx->stream));
-    GDR_CUDA(cudaStreamSynchronize(ctx->stream));
+    bool tc_failed;
+    const ColState out = fetch_state(ctx, d.st, tc_failed);
     if (out.err) throw gdr_error((gdr_status)out.err, "harmonic Ritz restart failed");
+    if (tc_failed) tc_fail(ctx);
   });
 }
 
@@ -932,8 +920,18 @@ gdr_status gdr_barrier_selftest(gdr_ctx* ctx, int rounds, int phantom) {
     GDR_REQUIRE(rounds >= 1 && rounds <= 1000000, "rounds must be in [1, 1e6]");
     r = barrier_selftest(ctx, rounds, phantom ? 1 : 0);
     if (r != GDR_OK) ctx->err = "grid barrier gave up (spin bound reached)";
+    else tc_check(ctx);
   });
   return g != GDR_OK ? g : r;
+}
+
+gdr_status gdr_tc_wait_selftest(gdr_ctx* ctx) {
+  if (!ctx) return GDR_EINVAL;
+  return guarded(ctx, [&] {
+    GDR_CUDA(cudaSetDevice(ctx->device));
+    GDR_REQUIRE(ctx->tc_err, "the tensor-core kernels are not available on this device");
+    tc_wait_selftest(ctx);
+  });
 }
 
 gdr_status gdr_basis_update(gdr_ctx* ctx, gdr_prec prec, long n, int nv, void* V, const double* C, int nout, int nx,

@@ -168,6 +168,14 @@ bool tc_proj_dot(gdr_ctx* ctx, long n, const c64* V, long ldv, int nv, const c64
 // (nothing launched) when it does not apply.
 bool tc_proj_update(gdr_ctx* ctx, long n, const c64* V, long ldv, int nv, const c128* C, long ccs, int rmode, c64* R,
                     long ldr, int ncol, const ColState* st, int* err, double prof_bytes);
+// After a wait: tc_failed tells whether a tensor-core kernel queued since the last report gave up
+// (its result is then incomplete); tc_fail clears the word and throws GDR_ETIMEOUT; tc_check does
+// both.  Every entry point that synchronises goes through one of them, so that a
+// gdr_basis_update, which does not wait itself, is reported by the next such call.
+ColState fetch_state(gdr_ctx* ctx, const ColState* st, bool& tc_failed);
+[[noreturn]] void tc_fail(gdr_ctx* ctx);
+void tc_check(gdr_ctx* ctx);
+void tc_wait_selftest(gdr_ctx* ctx);
 // GMRES-DR restart on the tensor cores (split TF32, as tc_proj_update): for ncol batch columns
 // with their own bases (stride vcs, lengths nvec), V[:, 0:nout] <- V C[:, 0:nout] in place and
 // X[:, i] += V C[:, nout + i] for i < nx (FP64); C has nv rows at stride ldc, ccs per column.

@@ -118,10 +118,10 @@ extern "C" gdr_status gdr_dense_gmres_sh_noalloc(gdr_ctx* ctx, int m, int ns, co
     dense_cycle(ctx, d);
     GDR_CUDA(cudaMemcpy2DAsync(D, m * sizeof(c128), Cf, (m + 1) * sizeof(c128), m * sizeof(c128), ns,
                                cudaMemcpyDeviceToDevice, ctx->stream));
-    ColState out;
-    GDR_CUDA(cudaMemcpyAsync(&out, st, sizeof(out), cudaMemcpyDeviceToHost, ctx->stream));
-    GDR_CUDA(cudaStreamSynchronize(ctx->stream));
+    bool tc_failed;
+    const ColState out = fetch_state(ctx, st, tc_failed);
     if (out.err) throw gdr_error((gdr_status)out.err, "singular reduced system");
+    if (tc_failed) tc_fail(ctx);
     return GDR_OK;
   } catch (const gdr_error& e) {
     ctx->err = e.what();

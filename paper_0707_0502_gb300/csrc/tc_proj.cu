@@ -972,6 +972,54 @@ bool tc_restart(gdr_ctx* ctx, long n, int ncol, c64* V, long ldv, long vcs, int 
   return true;
 }
 
+// ------------------------------------------------------- waits that gave up
+
+// Wait for the stream and for the word that a kernel above sets when one of its waits gives up,
+// and, when given, for a batch's first column state -- behind the queued kernels, through the
+// context's pinned memory.
+ColState fetch_state(gdr_ctx* ctx, const ColState* st, bool& tc_failed) {
+  struct Host {
+    ColState st;
+    int err;
+  };
+  Host* h = static_cast<Host*>(ctx->host_status(sizeof(Host)));
+  *h = Host{};
+  if (st) GDR_CUDA(cudaMemcpyAsync(&h->st, st, sizeof(ColState), cudaMemcpyDeviceToHost, ctx->stream));
+  if (ctx->tc_err) GDR_CUDA(cudaMemcpyAsync(&h->err, ctx->tc_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  GDR_CUDA(cudaStreamSynchronize(ctx->stream));
+  tc_failed = h->err != 0;
+  return h->st;
+}
+
+void tc_fail(gdr_ctx* ctx) {
+  GDR_CUDA(cudaMemsetAsync(ctx->tc_err, 0, sizeof(int), ctx->stream));
+  GDR_CUDA(cudaStreamSynchronize(ctx->stream));
+  throw gdr_error(GDR_ETIMEOUT,
+                  "a tensor-core wait gave up, in this call or in a gdr_basis_update queued since the last call that "
+                  "synchronised");
+}
+
+void tc_check(gdr_ctx* ctx) {
+  bool failed;
+  fetch_state(ctx, nullptr, failed);
+  if (failed) tc_fail(ctx);
+}
+
+namespace {
+// one wait for an arrival that never comes, ended by its limit (about a second)
+__global__ void tc_wait_selftest_kernel(int* err) {
+  __shared__ __align__(8) uint64_t bar;
+  int own = 0;
+  mbar_init(&bar, 1);
+  if (!mbar_wait(&bar, 0, &own)) atomicExch(err, 1);
+}
+}  // namespace
+
+void tc_wait_selftest(gdr_ctx* ctx) {
+  tc_wait_selftest_kernel<<<1, 1, 0, ctx->stream>>>(ctx->tc_err);
+  GDR_LAUNCHED(ctx);
+}
+
 void tc_proj_init(gdr_ctx* ctx) {
   ctx->tc_ok = false;
   if (!encoder()) return;
