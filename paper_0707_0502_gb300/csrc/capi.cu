@@ -3,6 +3,7 @@
 // this boundary.
 #include <array>
 #include <chrono>
+#include <cmath>
 #include <cstring>
 #include <type_traits>
 
@@ -746,7 +747,8 @@ gdr_status gdr_arnoldi_cycle(gdr_ctx* ctx, const gdr_op* A, gdr_prec prec, void*
       s.active = 1;
       s.m_eff = m;
       GDR_CUDA(cudaMemcpyAsync(b.st, &s, sizeof(s), cudaMemcpyHostToDevice, ctx->stream));
-      if (std::is_same<R, float>::value && !(flags & GDR_FLAG_CGS2)) {
+      const bool dcgs2 = std::is_same<R, float>::value && !(flags & GDR_FLAG_CGS2);
+      if (dcgs2) {
         arnoldi_dcgs2<R>(ctx, A, b, j0, m);
       } else {
         cx<R>* wl = nullptr;
@@ -765,7 +767,10 @@ gdr_status gdr_arnoldi_cycle(gdr_ctx* ctx, const gdr_op* A, gdr_prec prec, void*
       const ColState out = fetch_state(ctx, b.st, tc_failed);
       if (m_eff) *m_eff = out.broke ? out.m_eff : m;
       if (out.broke) {  // columns the breakdown left: 0 (here, not by clearing the basis before every cycle)
-        const int c0 = std::max(out.m_eff, j0 + 1);
+        // a step of the delayed form that met a non-finite w = A u stops before it makes v_j of u
+        // (its m_eff counts the step): that column is left, too
+        const bool met = dcgs2 && out.nan && !std::isfinite(out.wnorm0);
+        const int c0 = std::max(out.m_eff - (met ? 1 : 0), j0 + 1);
         if (c0 <= m) {
           GDR_CUDA(cudaMemsetAsync(static_cast<cx<R>*>(V) + (long)c0 * n, 0, sizeof(cx<R>) * n * (m + 1 - c0),
                                    ctx->stream));
