@@ -210,7 +210,8 @@ long gdr_op_n(const gdr_op *op);
 
 /* Matvec (step a1 / a2): Y[:,c] = (A - sigma_c I) X[:,c], c < ncol, in the
  * precision `prec` (FP64: X, Y are c128; MIXED: X, Y are complex64, interleaved
- * floats).  sigma: host c128[ncol].  Leading dimension n.  A CSR batch: column c
+ * floats).  sigma: host c128[ncol] (under stream capture read again at each
+ * replay).  Leading dimension n.  A CSR batch: column c
  * belongs to problem c, ncol <= the number of problems.  Asynchronous. */
 gdr_status gdr_op_apply(gdr_ctx *ctx, const gdr_op *A, gdr_prec prec, int ncol, const double *sigma,
                         const void *X, void *Y);

@@ -681,8 +681,6 @@ static void wilson_order_launch(gdr_ctx* ctx, long V, int cols, const T* in, lon
     wilson_order_elem_kernel<K><<<grid, 256, 0, ctx->stream>>>(V, reinterpret_cast<const float2*>(in), ldi * K,
                                                                reinterpret_cast<float2*>(out), ldo * K, to_lib ? 1 : 0);
     GDR_LAUNCHED(ctx);
-    if (sdst)
-      GDR_CUDA(cudaMemcpyAsync(sdst, sg.v, sizeof(c128) * sg.n, cudaMemcpyHostToDevice, ctx->stream));
     return;
   }
   wilson_order_kernel<T><<<dim3((unsigned)((V + OS - 1) / OS), (unsigned)cols), 128, 0, ctx->stream>>>(
@@ -711,13 +709,21 @@ void op_order(gdr_ctx* ctx, const gdr_op* A, int cols, const T* in, long ldi, T*
 template void op_order<c128>(gdr_ctx*, const gdr_op*, int, const c128*, long, c128*, long, bool);
 template void op_order<c64>(gdr_ctx*, const gdr_op*, int, const c64*, long, c64*, long, bool);
 
+static bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();
+  return st != cudaStreamCaptureStatusNone;
+}
+
 // Matvec at the C interface (user's vectors, shifts on the host).  Wilson: one reordering pass
 // into the library's order (it also brings up to 16 shifts, which saves their copy), then the
-// matvec, which stores site-major.
+// matvec, which stores site-major.  A captured call copies the shifts from the user's array, so
+// that a replay reads what stands there then.
 template <typename R>
 void op_apply_user(gdr_ctx* ctx, const gdr_op* A, int ncol, const double* sigma, const cx<R>* X, cx<R>* Y) {
   c128* sd = ctx->get<c128>("apply.sigma", (size_t)std::max(ncol, 16));
-  const bool wil = A->kind == OP_WILSON, by_value = wil && ncol <= 16;
+  const bool wil = A->kind == OP_WILSON;
+  const bool by_value = wil && ncol <= 16 && aligned16(X, 0, 1) && !capturing(ctx->stream);
   if (!by_value) GDR_CUDA(cudaMemcpyAsync(sd, sigma, sizeof(c128) * ncol, cudaMemcpyHostToDevice, ctx->stream));
   if (!wil) {
     op_apply<R>(ctx, A, ncol, sd, X, A->n, Y, A->n, nullptr, 0);
