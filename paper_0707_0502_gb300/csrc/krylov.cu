@@ -575,13 +575,10 @@ __global__ void __launch_bounds__(CT) combine_kernel(long n, cx<R>* V, long ldv,
   if (rr >= rows) return;
   const long row = r0 + rr;
   for (int o = threadIdx.x / CR; o < ntot; o += CT / CR) {
-    cx<R> acc = {0, 0};
+    CSum<R> sum;
     const cx<R>* co = cf + (long)o * nv;
-    if constexpr (sizeof(R) == 8) {
-      for (int i = 0; i < nv; ++i) acc = cfma(acc, tile[(long)i * CR + rr], co[i]);
-    } else {
-      for (int i = 0; i < nv; ++i) acc += tile[(long)i * CR + rr] * co[i];
-    }
+    for (int i = 0; i < nv; ++i) sum.mac(tile[(long)i * CR + rr], co[i]);
+    const cx<R> acc = sum.value();
     if (o < nout) {
       Vc[(long)o * ldv + row] = acc;
     } else if (o < nout + nx) {
@@ -625,31 +622,30 @@ __global__ void __launch_bounds__(256) combine_rows_kernel(long n, const cx<R>* 
   __syncthreads();
   const cx<R>* Vc = V + (c / vpp) * vcs;
   for (long row = blockIdx.x * 256L + threadIdx.x; row < n; row += (long)gridDim.x * 256) {
-    cx<R> acc[NO];
-#pragma unroll
-    for (int o = 0; o < NO; ++o) acc[o] = {0, 0};
+    CSum<R> acc[NO];
 #pragma unroll 4
     for (int i = 0; i < nv; ++i) {
       const cx<R> v = Vc[(long)i * ldv + row];
 #pragma unroll
       for (int o = 0; o < NO; ++o)
-        if (o < ntot) acc[o] = sizeof(R) == 8 ? cfma(acc[o], v, cf[o * nv + i]) : acc[o] + v * cf[o * nv + i];
+        if (o < ntot) acc[o].mac(v, cf[o * nv + i]);
     }
 #pragma unroll
     for (int o = 0; o < NO; ++o) {
       if (o >= ntot) break;
+      const cx<R> a = acc[o].value();
       if (o < nx) {
         if (Xf) {  // correction accumulated in the vectors' precision
           cx<R>* fp = Xf + c * xcs + (long)o * ldx + row;
-          *fp = *fp + acc[o];
+          *fp = *fp + a;
         } else {
           c128* xp = X + c * xcs + (long)o * ldx + row;
-          *xp = *xp + up(acc[o]);
+          *xp = *xp + up(a);
         }
       } else {
         cx<R>* rp = Rv + c * rcs + row;
-        if (rmode == 1) *rp = acc[o];
-        else *rp = *rp + acc[o];
+        if (rmode == 1) *rp = a;
+        else *rp = *rp + a;
       }
     }
   }
@@ -693,18 +689,17 @@ __global__ void __launch_bounds__(CT) combine_shared_kernel(long n, const cx<R>*
     // the CT / CR = 4 thread groups of a row take interleaved pairs
     const long P = (long)ncol * ntot;
     for (long p0 = threadIdx.x / CR; p0 < P; p0 += 4 * (CT / CR)) {
-      cx<R> acc[4];
+      CSum<R> acc[4];
       const cx<R>* co[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const long pq = min(p0 + (long)q * (CT / CR), P - 1);
         co[q] = cf + (pq / ntot) * per + (pq % ntot) * nv;
-        acc[q] = {0, 0};
       }
       for (int i = 0; i < nv; ++i) {
         const cx<R> t = tile[(long)i * CR + rr];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q] = sizeof(R) == 8 ? cfma(acc[q], t, co[q][i]) : acc[q] + t * co[q][i];
+        for (int q = 0; q < 4; ++q) acc[q].mac(t, co[q][i]);
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -712,13 +707,14 @@ __global__ void __launch_bounds__(CT) combine_shared_kernel(long n, const cx<R>*
         if (pq >= P) break;
         const int c = (int)(pq / ntot), o = (int)(pq % ntot);
         if (st && !st[c].active) continue;
+        const cx<R> a = acc[q].value();
         if (o < nx) {
           c128* xp = X + c * xcs + (long)o * ldx + row;
-          *xp = *xp + up(acc[q]);
+          *xp = *xp + up(a);
         } else {
           cx<R>* rp = Rv + c * rcs + row;
-          if (rmode == 1) *rp = acc[q];
-          else *rp = *rp + acc[q];
+          if (rmode == 1) *rp = a;
+          else *rp = *rp + a;
         }
       }
     }
@@ -787,10 +783,16 @@ __global__ void __launch_bounds__(DS_W * 32) gs_dot_shared_kernel(long n, const 
 #pragma unroll
     for (int i = 0; i < NVM; ++i) {
       if (i >= nv) break;
+      if constexpr (sizeof(R) == 8) {
+        // a tile's four products as one FMA chain, then a single rounding of the long sum (two
+        // accumulators per vector would not fit the registers): 9 FP64 instructions a part, not 12
+        cx<R> t = cmulc(vt[i * DS_TR + lane], rv[0]);
 #pragma unroll
-      for (int q = 0; q < DS_EPL; ++q) {
-        const cx<R> v = vt[i * DS_TR + lane + 32 * q];
-        acc[i] = sizeof(R) == 8 ? cfma(acc[i], conj(v), rv[q]) : acc[i] + cmulc(v, rv[q]);
+        for (int q = 1; q < DS_EPL; ++q) t = cfma(t, conj(vt[i * DS_TR + lane + 32 * q]), rv[q]);
+        acc[i] += t;
+      } else {
+#pragma unroll
+        for (int q = 0; q < DS_EPL; ++q) acc[i] += cmulc(vt[i * DS_TR + lane + 32 * q], rv[q]);
       }
     }
     if (++cnt == DS_FL) {
@@ -849,7 +851,7 @@ __global__ void axpy_cols_kernel(long n, const c128* a, const c128* S, long ssc,
   const int c = blockIdx.y;
   const c128 ac = a[c];
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-    X[c * xcs + i] = cfma(X[c * xcs + i], ac, S[c * ssc + i]);
+    X[c * xcs + i] += ac * S[c * ssc + i];
 }
 __global__ void scal_cols_kernel(long n, const c128* a, c128* X, long xcs) {
   const int c = blockIdx.y;

@@ -85,7 +85,7 @@ __global__ void correct_kernel(long n, int ns, const c128* gam, const c128* S, l
   if (i == 0) return;
   const c128 g = gam[p];
   for (long r = blockIdx.x * (long)blockDim.x + threadIdx.x; r < n; r += (long)gridDim.x * blockDim.x)
-    X[(long)p * ldx + r] = cfma(X[(long)p * ldx + r], g, S[(long)i * lds + r]);
+    X[(long)p * ldx + r] += g * S[(long)i * lds + r];
 }
 
 // Residuals after the correction, without a matvec: with s_i = s~_i / (1 - gs_i) and
@@ -106,7 +106,7 @@ __global__ void corrected_resid_kernel(long n, int ns, const c128* gam, const c1
   c128* ro = Rout + (long)p * ld;
   const c128* rs = Rs + (long)i * ld;
   for (long r = blockIdx.x * (long)blockDim.x + threadIdx.x; r < n; r += (long)gridDim.x * blockDim.x)
-    ro[r] = i > 0 ? cfnma(ri[r], f, v[r] - rs[r]) : ri[r];
+    ro[r] = i > 0 ? ri[r] - f * (v[r] - rs[r]) : ri[r];
 }
 
 // Related right-hand sides (Sec. 5, eqs. relrhs1-relrhs2).  M is the j x (j+1)
