@@ -230,6 +230,13 @@ DEV void warp_givens_qr(c128* A, int lda, int rows, int j0, int cols, int ntot) 
 // pass), then, with v = x scal known, A[:, c] -= x (scal f_c), f_c = conj(tau) (A[j, c] +
 // conj(scal) d_c).  The scalars are formed by every thread for itself, two barriers a column.
 // A 41 x 40 system with six shifts (two such solves one after the other): 1,110 us before.
+//
+// Every update forms its product first (A -= x h with one rounding of A): an entry passes through
+// up to 96 of them, and as FMA chains, two roundings each, they cost y and s 10 to 25% in error.
+DEV double quot(double a, double b, double ib) {  // a / b, ib = 1 / b rounded
+  const double t = a * ib;
+  return fma(fma(-b, t, a), ib, t);
+}
 template <int L>
 DEV double reflect_r(c128* A, int lda, int j, int last, int ntot, double* norm_s, c128* keep) {  // returns R[j, j]
   const int g = threadIdx.x / L, l = threadIdx.x % L, NG = DT / L;
@@ -258,12 +265,16 @@ DEV double reflect_r(c128* A, int lda, int j, int last, int ntot, double* norm_s
     if (keep && threadIdx.x == 0) keep[0] = keep[1] = {0, 0};
     return alpha.x;
   }
-  const double n2 = norm2(alpha) + s, inv = rsqrt_nr(n2);
-  const double beta = -copysign(n2 * inv, alpha.x), ib = -copysign(inv, alpha.x);
-  const c128 ctau = {(beta - alpha.x) * ib, alpha.y * ib};  // conj(tau)
+  // sqrt, 1/beta and the quotients each with one Newton correction of its residual, by which they
+  // are as good as the operations themselves (uncorrected the reflectors are unitary to a few
+  // units of the last place only, and y's error at m = 80 was 10% larger)
+  const double n2 = norm2(alpha) + s, inv0 = rsqrt_nr(n2), root0 = n2 * inv0;
+  const double root = fma(fma(-root0, root0, n2), 0.5 * inv0, root0), inv = fma(fma(-root, inv0, 1.0), inv0, inv0);
+  const double beta = -copysign(root, alpha.x), ib = -copysign(inv, alpha.x);
+  const c128 ctau = {quot(beta - alpha.x, beta, ib), quot(alpha.y, beta, ib)};  // conj(tau)
   const c128 ab = {alpha.x - beta, alpha.y};
-  const double rd = 1.0 / norm2(ab);
-  const c128 scal = {ab.x * rd, -ab.y * rd};
+  const double nab = norm2(ab), rd = 1.0 / nab;
+  const c128 scal = {quot(ab.x, nab, rd), quot(-ab.y, nab, rd)};
   if (keep && threadIdx.x == 0) {
     keep[0] = ctau;
     keep[1] = scal;
@@ -278,7 +289,7 @@ DEV double reflect_r(c128* A, int lda, int j, int last, int ntot, double* norm_s
     if (on) {
       f = ctau * cfma(col[j], conj(scal), dc[p]);
       const c128 h = scal * f;
-      for (int i = j + 1 + l; i <= last; i += L) col[i] = cfnma(col[i], x[i], h);
+      for (int i = j + 1 + l; i <= last; i += L) col[i] -= x[i] * h;
     }
     __syncwarp();  // the group's lanes have read col[j]
     if (on && l == 0) col[j] -= f;
@@ -332,7 +343,7 @@ DEV void apply_kept(const c128* A, int lda, int rows, int cols, int kfull, const
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       if (32 * q > last) break;
-      v[q] = cfnma(v[q], xi[q], g);
+      v[q] -= xi[q] * g;
       if (lane + 32 * q == j) v[q] -= f;
     }
   }
@@ -367,7 +378,8 @@ DEV bool fast_backsolve(const c128* A, int lda, int nsz, c128* y, c128* rinv, Sh
       const c128 xj = y[j] * rinv[j];
       __syncwarp();
       if (threadIdx.x == 0) y[j] = xj;
-      for (int i = threadIdx.x; i < j; i += 32) y[i] = cfnma(y[i], A[i + (long)j * lda], xj);
+      // the product first: one rounding of y_i per term
+      for (int i = threadIdx.x; i < j; i += 32) y[i] -= A[i + (long)j * lda] * xj;
       __syncwarp();
     }
   }
@@ -543,10 +555,10 @@ DEV void base_ls(const DenseCycle& d, int c, c128* A, Sh& sh) {
     c128 v = {0, 0};
     if (!broke && i <= me) {
       v = cv[i];
-      for (int j = 0; j < me; ++j) {
+      for (int j = 0; j < me; ++j) {  // s is small: what is left of c keeps shrinking, and so do the roundings
         c128 hij = H[i + (long)j * (m + 1)];
         if (i == j) hij -= sig;
-        v = cfnma(v, hij, y[j]);
+        v -= hij * y[j];
       }
     }
     s[i] = v;

@@ -130,3 +130,28 @@ def test_least_squares_residual(ctx):
     y, s = _reduced(ctx, H, c)
     assert np.abs(y - (1 + 1j)).max() < 1e-14
     _check(s[m], _exact([(c[m], 1 + 0j)] + [(-H[m, j], y[j]) for j in range(m)]), m + 1)
+
+
+@pytest.mark.parametrize("ns", [2, 9])
+def test_reflected_right_hand_side(ctx, ns):
+    """beta_new of a shift at which H is a unit matrix over a small last row t: m reflectors each take
+    t_j c_j from the last component of c, and beta_new (s_m - sum t_j s_j) = c_m - sum t_j c_j.
+    The base shift lies far away, so that s differs from c in the last component only.  (Two
+    shifts: one cluster; nine: two launches.)"""
+    m = 80
+    H = np.eye(m + 1, m, dtype=complex)
+    H[m] = -BIG - 0.5j * SMALL
+    c = np.full(m + 1, 1 + 1j)
+    c[m] = 1
+    z = lambda *sh: torch.zeros(sh, dtype=torch.complex128, device="cuda")
+    D, s, bn = z(ns, m), z(m + 1), z(ns)
+    g.gdr_dense_gmres_sh(ctx, m, [-1023.0] + [0.0] * (ns - 1), dev(np.ascontiguousarray(H.T)), dev(c),
+                         dev(np.ones(ns, complex)), D, s, bn, torch.zeros(ns, dtype=torch.float64, device="cuda"))
+    s, bn = host(s), host(bn)
+    assert abs(s[m] - 1) < 1e-14 and np.abs(s[:m]).max() < 1e-12
+    num = _exact([(c[m], 1 + 0j)] + [(-H[m, j], c[j]) for j in range(m)])
+    den = _exact([(s[m], 1 + 0j)] + [(-H[m, j], s[j]) for j in range(m)])
+    d2 = den[0] ** 2 + den[1] ** 2
+    want = (num[0] * den[0] + num[1] * den[1]) / d2, (num[1] * den[0] - num[0] * den[1]) / d2
+    for b in bn[1:]:
+        _check(b, want, m + 10)   # ten more roundings for the quotient
