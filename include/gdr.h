@@ -418,8 +418,8 @@ gdr_status gdr_dense_restart(gdr_ctx *ctx, gdr_prec prec, int m, int k, const do
  * V (n x nv, `prec`) times coefficients C (c128 nv x (nout + nx)):
  * V[:, 0:nout] <- V C[:, 0:nout]  (in place, nout <= nv) and
  * X[:, i] += V C[:, nout + i] for i < nx (X c128 n x nx).
- * MIXED with 0 < nout and 26 <= nout + nx <= 64 (from 16 on with more than 60 vectors) runs on
- * the tensor cores (both factors split into two TF32 parts, FP32 accumulation: FP32
+ * MIXED with 0 < nout, nv >= 54 and 26 <= nout + nx <= 64 (from 16 on with more than 60 vectors)
+ * runs on the tensor cores (both factors split into two TF32 parts, FP32 accumulation: FP32
  * arithmetic's accuracy), below that on the CUDA cores in FP32; the call has no switch.
  * A tensor-core wait that gave up is reported by the next call that synchronises
  * (GDR_ETIMEOUT, V and X then unspecified). */

@@ -179,7 +179,8 @@ void tc_wait_selftest(gdr_ctx* ctx);
 // GMRES-DR restart on the tensor cores (split TF32, as tc_proj_update): for ncol batch columns
 // with their own bases (stride vcs, lengths nvec), V[:, 0:nout] <- V C[:, 0:nout] in place and
 // X[:, i] += V C[:, nout + i] for i < nx (FP64); C has nv rows at stride ldc, ccs per column.
-// False (nothing launched) when its coefficients do not fit in shared memory.
+// False (nothing launched) where the CUDA-core form is the better one (fewer than 54 vectors, few
+// outputs: see there) or its coefficients do not fit in shared memory.
 bool tc_restart(gdr_ctx* ctx, long n, int ncol, c64* V, long ldv, long vcs, int nv, const c128* C, long ldc, long ccs,
                 int nout, int nx, c128* X, long ldx, long xcs, const ColState* st, const int* nvec, int* err);
 

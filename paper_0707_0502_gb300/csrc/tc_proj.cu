@@ -343,6 +343,7 @@ constexpr int TU_DW = 256;          // tensor-memory columns of one accumulator 
 constexpr int TU_DLO = 128;         // ... and its first column of the products with a lo part
 constexpr int TU_SC = 16;           // columns that a group of four epilogue warps stages at a time
 constexpr int TU_MAXNV = 48;        // basis vectors of the residual update
+constexpr int TU_MINNV = 54;        // fewest of the restart
 constexpr int TU_STAGES = 2;        // K atoms of A, one per group of four writer warps
 constexpr int TU_MAXOUT = 64;       // outputs of the restart: hi and lo parts of B side by side in one MMA (N = 128)
 constexpr int TU_RAW_ROW = 512;     // bytes of one vector's rows in `raw`
@@ -946,7 +947,10 @@ bool tc_restart(gdr_ctx* ctx, long n, int ncol, c64* V, long ldv, long vcs, int 
   //   41 vectors, 20 outputs  10.8 -> 10.9 / 23.0 -> 25.1 / 233 -> 242;  26 outputs 1.06 / 1.07 / 1.13x
   //   51 vectors, 20 outputs  0.86 / 0.93 / 0.99x;                       26 outputs 1.04 / 1.08 / 1.18x
   //   61 vectors, 10 outputs  0.99 / 0.76 / 0.87x;                       15 outputs 1.09 / 1.09 / 1.17x
-  if (nn < (nv > 60 ? 16 : 26)) return false;
+  // And the error: each MMA truncates where an FP32 FMA rounds, so this form's is about 1.4e-7 of
+  // the result (rms) at any basis size, the CUDA cores' grows with the vectors: 1.04e-7 at 26, 1.25 at
+  // 41, 1.38 at 51, 1.41 at 54 (here 1.36), 1.49 at 61 (1.41), 1.69 at 81 (1.41).
+  if (nv < TU_MINNV || nn < (nv > 60 ? 16 : 26)) return false;
   if (nv < 1 || nv > GDR_MAX_M + 1 || nn > TU_MAXOUT || !ctx->tc_ok || !ctx->tc_update_ok ||
       tc_combine_smem(a.ka, (nn + 15) / 16 * 16, TU_MINRAW, 1) > ctx->tc_combine_smem)
     return false;
