@@ -301,6 +301,9 @@ struct KProf {
       idx = (int)c->prof_pending.size() - 1;
     }
   }
+  void rename(const char* name) {
+    if (idx >= 0) ctx->prof_pending[idx].name = name;
+  }
   ~KProf() {
     if (idx >= 0) cudaEventRecord(ctx->prof_pending[idx].b, ctx->stream);
   }

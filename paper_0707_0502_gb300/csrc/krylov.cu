@@ -1144,8 +1144,10 @@ void combine(gdr_ctx* ctx, long n, int ncol, cx<R>* V, long ldv, long vcs, int n
                                                  (rmode == 2 ? 2.0 : (rmode == 1 ? 1.0 : 0.0)) * sizeof(cx<R>))));
   if (std::is_same<R, float>::value && nout > 0 && rmode == 0 && vpp == 1 && ctx->tc_proj && ctx->tc_err &&
       tc_restart(ctx, n, ncol, reinterpret_cast<c64*>(V), ldv, vcs, nv, C, ldc, ccs, nout, nx, X, ldx, xcs, st, nvec,
-                 ctx->tc_err))
+                 ctx->tc_err)) {
+    kp.rename("tc_restart_c64");
     return;
+  }
   combine_kernel<R><<<grid, CT, smem, ctx->stream>>>(n, V, ldv, vcs, nv, C, ldc, ccs, nout, nx, rmode, X, ldx, xcs,
                                                      Rv, rcs, st, nvec, vpp, Xf);
   GDR_LAUNCHED(ctx);
