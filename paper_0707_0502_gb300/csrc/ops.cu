@@ -132,7 +132,7 @@ __global__ void csr_batch_kernel(const long* __restrict__ rp_off, const long* __
 
 // ---------------------------------------------------------- Wilson kernel
 
-// Site-major output (out_sm: the matvec of the C interface, whose vectors are site-major):
+// Site-major output (OUT_SM: the matvec of the C interface, whose vectors are site-major):
 // a warp's 32 sites are 32 x 12 consecutive elements of the result, so the warp passes its
 // spinors through shared memory and stores them contiguously -- the separate reordering pass
 // over the result (one read and one write of it) is not needed.  The dynamic shared memory
@@ -178,23 +178,23 @@ constexpr int wilson_min_blocks(int nt) {
   return (sizeof(R) == 4 ? 768 : 512) / nt;
 }
 
-template <typename R, typename LT, int NT>
+template <typename R, typename LT, int NT, bool OUT_SM>
 __global__ void __launch_bounds__(NT, wilson_min_blocks<R>(NT)) wilson_kernel(const LT* __restrict__ links, int Lx, int Ly, int Lz, int Lt,
                                                    double diag_a, const c128* __restrict__ sigma,
                                                    const cx<R>* __restrict__ X, long ldx, cx<R>* __restrict__ Y,
                                                    long ldy, const cx<R>* __restrict__ B, long ldb,
                                                    const int* __restrict__ run, int run_stride, int cpp,
                                                    const double* __restrict__ xs, int xs_stride, int ncol,
-                                                   int col_inner, int out_sm) {
+                                                   int col_inner) {
   const long V = (long)Lx * Ly * Lz * Lt;
   long tile;
   int c;
   tile_col(ncol, col_inner, tile, c);
   long site = tile * NT + threadIdx.x;
-  pdl_wait();
+  if constexpr (OUT_SM) pdl_wait();
   if (run && !run[(long)c * run_stride]) return;
   if (site >= V) {  // a warp that stores together keeps all its lanes
-    if (!out_sm || (site & ~31L) >= V) return;
+    if (!OUT_SM || (site & ~31L) >= V) return;
     site = V - 1;
   }
   const cx<R>* x = X + c * ldx;
@@ -245,10 +245,10 @@ __global__ void __launch_bounds__(NT, wilson_min_blocks<R>(NT)) wilson_kernel(co
       v0 = out(p.s[2 * i], acc.s[2 * i], {0, 0}, false);
       v1 = out(p.s[2 * i + 1], acc.s[2 * i + 1], {0, 0}, false);
     }
-    if (out_sm) stage_pair<R>(i, v0, v1);
+    if (OUT_SM) stage_pair<R>(i, v0, v1);
     else store_pair<R>(y, V, site, i, v0, v1);
   }
-  if (out_sm) store_staged<R>(y, V, tile * NT);
+  if (OUT_SM) store_staged<R>(y, V, tile * NT);
 }
 
 // Small lattices: a block takes 32 sites and warp w computes the two hops in
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(NT, wilson_min_blocks<R>(NT)) wilson_kernel(co
 // dependency chain), the four partial spinors are summed through shared memory
 // and the output, with the diagonal term, is written one component per thread
 // (coalesced).  Used when one thread per site cannot fill the GPU.
-template <typename R, typename LT>
+template <typename R, typename LT, bool OUT_SM>
 __global__ void __launch_bounds__(128) wilson_split_kernel(const LT* __restrict__ links, int Lx, int Ly, int Lz,
                                                           int Lt, double diag_a, const c128* __restrict__ sigma,
                                                           const cx<R>* __restrict__ X, long ldx,
@@ -264,13 +264,13 @@ __global__ void __launch_bounds__(128) wilson_split_kernel(const LT* __restrict_
                                                           const cx<R>* __restrict__ B, long ldb,
                                                           const int* __restrict__ run, int run_stride, int cpp,
                                                           const double* __restrict__ xs, int xs_stride, int ncol,
-                                                          int col_inner, int out_sm) {
+                                                          int col_inner) {
   __shared__ cx<R> part[4][32][13];  // odd row length: conflict-free in both phases
   const long V = (long)Lx * Ly * Lz * Lt;
   long tile;
   int c;
   tile_col(ncol, col_inner, tile, c);
-  pdl_wait();
+  if constexpr (OUT_SM) pdl_wait();
   if (run && !run[(long)c * run_stride]) return;
   const int mu = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long site0 = tile * 32L, site = site0 + lane;
@@ -299,14 +299,14 @@ __global__ void __launch_bounds__(128) wilson_split_kernel(const LT* __restrict_
   // output element q: pair q / 64, site q % 64 / 2, half q % 2 (64 consecutive elements of a
   // pair); site-major output: site q / 12, component q % 12
   for (int q = threadIdx.x; q < 6 * 64; q += 128) {
-    const int pr = out_sm ? (q % 12) >> 1 : q >> 6, sl = out_sm ? q / 12 : (q & 63) >> 1, hf = q & 1;
+    const int pr = OUT_SM ? (q % 12) >> 1 : q >> 6, sl = OUT_SM ? q / 12 : (q & 63) >> 1, hf = q & 1;
     const int comp = 2 * pr + hf;
     if (site0 + sl >= V) continue;
     const cx<R> h = part[0][sl][comp] + part[1][sl][comp] + part[2][sl][comp] + part[3][sl][comp];
     const long e = 2 * ((long)pr * V + site0 + sl) + hf;
     cx<R> v = sc * (dg * x[e] - h);
     if (b) v = b[e] - v;
-    y[out_sm ? site0 * 12 + q : e] = v;
+    y[OUT_SM ? site0 * 12 + q : e] = v;
   }
 }
 
@@ -315,21 +315,21 @@ __global__ void __launch_bounds__(128) wilson_split_kernel(const LT* __restrict_
 // with itself and stored once.  Same operator and output as wilson_kernel.
 // Registers are capped for 16 resident warps per SM (128 registers): with 12 warps and no
 // cap (168 registers) the same kernel was 17% slower at 24^3x32, 12 columns.
-template <typename LT, int NT>
+template <typename LT, int NT, bool OUT_SM>
 __global__ void __launch_bounds__(NT, 512 / NT) wilson_pair_kernel(
     const LT* __restrict__ links, int Lx, int Ly, int Lz, int Lt, double diag_a, const c128* __restrict__ sigma,
     const c64* __restrict__ X, long ldx, c64* __restrict__ Y, long ldy, const c64* __restrict__ B, long ldb,
     const int* __restrict__ run, int run_stride, int cpp, const double* __restrict__ xs, int xs_stride, int ncol,
-    int col_inner, int out_sm) {
+    int col_inner) {
   const long V = (long)Lx * Ly * Lz * Lt;
   const int npair = (ncol + 1) / 2;
   long tile;
   int cp;
   tile_col(npair, col_inner, tile, cp);
   long site = tile * NT + threadIdx.x;
-  pdl_wait();
+  if constexpr (OUT_SM) pdl_wait();
   if (site >= V) {
-    if (!out_sm || (site & ~31L) >= V) return;
+    if (!OUT_SM || (site & ~31L) >= V) return;
     site = V - 1;
   }
   const int c0 = 2 * cp, c1 = min(2 * cp + 1, ncol - 1);
@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) wilson_pair_kernel(
     f2_unpack(v[0].im, a0i, a1i);
     f2_unpack(v[1].re, b0r, b1r);
     f2_unpack(v[1].im, b0i, b1i);
-    if (out_sm) {  // column c0 now, c1's values kept for a second round through the stage
+    if (OUT_SM) {  // column c0 now, c1's values kept for a second round through the stage
       stage_pair<float>(i, {a0r, a0i}, {b0r, b0i});
       acc.s[2 * i] = v[0];
       acc.s[2 * i + 1] = v[1];
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) wilson_pair_kernel(
       if (st1) y1[i * V] = make_float4(a1r, a1i, b1r, b1i);
     }
   }
-  if (out_sm) {
+  if (OUT_SM) {
     if (st0) store_staged<float>(Y + c0 * ldy, V, tile * NT);
     if (!st1) return;
     __syncwarp();
@@ -513,19 +513,19 @@ static void csr_launch(gdr_ctx* ctx, const gdr_op* A, const VT* vals, const MvSh
   GDR_LAUNCHED(ctx);
 }
 
-template <typename R, typename LT>
+template <typename R, typename LT, bool OUT_SM>
 static void wilson_launch(gdr_ctx* ctx, const gdr_op* A, const LT* links, const MvShape& s, int ncol,
                           const c128* sigma, const cx<R>* X, long ldx, cx<R>* Y, long ldy, const cx<R>* B, long ldb,
-                          const int* run, int run_stride, int cpp, const double* xs, int xs_stride, int out_sm) {
+                          const int* run, int run_stride, int cpp, const double* xs, int xs_stride) {
   const int* d = A->dims;
-  auto stage = [&](int nt) { return out_sm ? (size_t)nt * 12 * sizeof(cx<R>) : (size_t)0; };
+  auto stage = [&](int nt) { return OUT_SM ? (size_t)nt * 12 * sizeof(cx<R>) : (size_t)0; };
   if constexpr (std::is_same<R, float>::value) {
     if (s.form == 2) {  // column pairs, packed FP32x2
       const int npair = (ncol + 1) / 2;
 #define GDR_WILSON_PAIR(NT)                                                                                          \
-  launch_pdl(out_sm != 0, wilson_pair_kernel<LT, NT>, tile_grid((A->V + NT - 1) / NT, npair, s.col_inner), NT, stage(NT), ctx->stream, \
+  launch_pdl(OUT_SM, wilson_pair_kernel<LT, NT, OUT_SM>, tile_grid((A->V + NT - 1) / NT, npair, s.col_inner), NT, stage(NT), ctx->stream, \
       links, d[0], d[1], d[2], d[3], A->diag_a, sigma, X, ldx, Y, ldy, B, ldb, run, run_stride, cpp, xs, xs_stride, \
-      ncol, s.col_inner, out_sm)
+      ncol, s.col_inner)
       if (s.threads == 64) GDR_WILSON_PAIR(64);
       else GDR_WILSON_PAIR(128);
 #undef GDR_WILSON_PAIR
@@ -534,14 +534,14 @@ static void wilson_launch(gdr_ctx* ctx, const gdr_op* A, const LT* links, const 
     }
   }
   if (s.form == 1) {
-    launch_pdl(out_sm != 0, wilson_split_kernel<R, LT>, tile_grid((A->V + 31) / 32, ncol, s.col_inner), 128, 0, ctx->stream,
+    launch_pdl(OUT_SM, wilson_split_kernel<R, LT, OUT_SM>, tile_grid((A->V + 31) / 32, ncol, s.col_inner), 128, 0, ctx->stream,
         links, d[0], d[1], d[2], d[3], A->diag_a, sigma, X, ldx, Y, ldy, B, ldb, run, run_stride, cpp, xs, xs_stride,
-        ncol, s.col_inner, out_sm);
+        ncol, s.col_inner);
   } else {
 #define GDR_WILSON_SITE(NT)                                                                                         \
-  launch_pdl(out_sm != 0, wilson_kernel<R, LT, NT>, tile_grid((A->V + NT - 1) / NT, ncol, s.col_inner), NT, stage(NT), ctx->stream, \
+  launch_pdl(OUT_SM, wilson_kernel<R, LT, NT, OUT_SM>, tile_grid((A->V + NT - 1) / NT, ncol, s.col_inner), NT, stage(NT), ctx->stream, \
       links, d[0], d[1], d[2], d[3], A->diag_a, sigma, X, ldx, Y, ldy, B, ldb, run, run_stride, cpp, xs, xs_stride, \
-      ncol, s.col_inner, out_sm)
+      ncol, s.col_inner)
     if (s.threads == 64) GDR_WILSON_SITE(64);
     else if (s.threads == 256) GDR_WILSON_SITE(256);
     else GDR_WILSON_SITE(128);
@@ -567,15 +567,19 @@ static void op_apply_launch(gdr_ctx* ctx, const gdr_op* A, int ncol, const c128*
       case 8: csr_launch<R, VT, 8>(ctx, A, vals, s, ncol, sigma, X, ldx, Y, ldy, B, ldb, run, run_stride, cpp, xs, xs_stride); break;
       default: csr_launch<R, VT, 1>(ctx, A, vals, s, ncol, sigma, X, ldx, Y, ldy, B, ldb, run, run_stride, cpp, xs, xs_stride); break;
     }
-  } else if constexpr (F64) {
-    wilson_launch<R, c128>(ctx, A, A->links128, s, ncol, sigma, X, ldx, Y, ldy, B, ldb, run, run_stride, cpp, xs,
-                           xs_stride, out_sm);
-  } else if (A->store == GDR_LINK_BF16) {
-    wilson_launch<R, __nv_bfloat162>(ctx, A, A->links16, s, ncol, sigma, X, ldx, Y, ldy, B, ldb, run, run_stride, cpp,
-                                     xs, xs_stride, out_sm);
   } else {
-    wilson_launch<R, c64>(ctx, A, A->links64, s, ncol, sigma, X, ldx, Y, ldy, B, ldb, run, run_stride, cpp, xs,
-                          xs_stride, out_sm);
+    auto launch = [&](const auto* links) {
+      using LT = std::remove_cv_t<std::remove_pointer_t<decltype(links)>>;
+      if (out_sm)
+        wilson_launch<R, LT, true>(ctx, A, links, s, ncol, sigma, X, ldx, Y, ldy, B, ldb, run, run_stride, cpp, xs,
+                                   xs_stride);
+      else
+        wilson_launch<R, LT, false>(ctx, A, links, s, ncol, sigma, X, ldx, Y, ldy, B, ldb, run, run_stride, cpp, xs,
+                                    xs_stride);
+    };
+    if constexpr (F64) launch(A->links128);
+    else if (A->store == GDR_LINK_BF16) launch(A->links16);
+    else launch(A->links64);
   }
 }
 
