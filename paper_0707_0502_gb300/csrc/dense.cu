@@ -241,7 +241,7 @@ template <int L>
 DEV double reflect_r(c128* A, int lda, int j, int last, int ntot, double* norm_s, c128* keep) {  // returns R[j, j]
   const int g = threadIdx.x / L, l = threadIdx.x % L, NG = DT / L;
   const c128* x = A + (long)j * lda;
-  constexpr int NP = 4;  // passes over the columns: at most GDR_MAX_M + 2 of them, 32 groups or more
+  constexpr int NP = 4;  // passes over the columns: at most GDR_MAX_M + 2 by 32 groups; one at L = 8 and 16
   c128 dc[NP];
 #pragma unroll
   for (int p = 0; p < NP; ++p) {
@@ -351,7 +351,7 @@ DEV void apply_kept(const c128* A, int lda, int rows, int cols, int kfull, const
 
 // QR of the GMRES recurrence matrix: Householder reflectors for its dense leading
 // block (columns < kfull - 1), Givens rotations for the Hessenberg columns after it.
-DEV void hess_qr(c128* A, int lda, int rows, int cols, int ntot, c128* tau, Sh& sh, int kfull) {
+DEV void hess_qr(c128* A, int lda, int rows, int cols, int ntot, Sh& sh, int kfull) {
   const int jd = max(0, min(cols, kfull - 1));
   cta_qr_r(A, lda, rows, jd, ntot, sh, kfull);
   warp_givens_qr(A, lda, rows, jd, cols, ntot);
@@ -528,19 +528,19 @@ DEV void base_ls(const DenseCycle& d, int c, c128* A, Sh& sh) {
   // square m x m Galerkin system
   const int rows = (broke || d.fom) ? me : me + 1;
   const int lda = odd_ld(rows);
-  c128* tau = A + (long)lda * (me + 1);
-  c128* y = tau + (me + 1);
+  c128* scr = A + (long)lda * (me + 1);
+  c128* y = scr + (me + 1);
   c128* rinv = y + (me + 1);
-  // complex64 basis, Hessenberg recurrence: FP32 least squares + refinement (tau as
-  // scratch), the FP64 form below when that is not trusted
+  // complex64 basis, Hessenberg recurrence: FP32 least squares + refinement (scr: its FP64
+  // residual), the FP64 form below when that is not trusted
   const bool done32 = d.ls32 && d.kfull <= 1 && !d.fom &&
-                      ls32_solve(H, m + 1, cv, sig, rows, me, reinterpret_cast<unsigned char*>(A), tau, y, sh);
+                      ls32_solve(H, m + 1, cv, sig, rows, me, reinterpret_cast<unsigned char*>(A), scr, y, sh);
   if (!done32) {
     load_shifted(A, lda, H, m + 1, rows, me, sig);
     for (int i = threadIdx.x; i < rows; i += DT) A[i + (long)me * lda] = cv[i];
     if (threadIdx.x == 0) sh.ibc[0] = 0;
     __syncthreads();
-    hess_qr(A, lda, rows, me, me + 1, tau, sh, d.kfull);
+    hess_qr(A, lda, rows, me, me + 1, sh, d.kfull);
     for (int i = threadIdx.x; i < me; i += DT) y[i] = A[i + (long)me * lda];
     __syncthreads();
     if (!fast_backsolve(A, lda, me, y, rinv, sh)) set_err(st, GDR_EBREAKDOWN);
@@ -623,12 +623,11 @@ DEV void shift_solve(const DenseCycle& d, int c, int i, c128* A, Sh& sh) {
     const int lda = odd_ld(me);
     load_shifted(A, lda, H, m + 1, me, me, sig);
     for (int r = threadIdx.x; r < me; r += DT) A[r + (long)me * lda] = cv[r];
-    c128* tau = A + (long)lda * (me + 1);
-    c128* y = tau + (me + 1);
+    c128* y = A + (long)lda * (me + 1);
     c128* rinv = y + (me + 1);
     if (threadIdx.x == 0) sh.ibc[0] = 0;
     __syncthreads();
-    hess_qr(A, lda, me, me, me + 1, tau, sh, d.kfull);
+    hess_qr(A, lda, me, me, me + 1, sh, d.kfull);
     for (int r = threadIdx.x; r < me; r += DT) y[r] = beta * A[r + (long)me * lda];
     __syncthreads();
     if (!fast_backsolve(A, lda, me, y, rinv, sh)) set_err(st, GDR_EBREAKDOWN);
@@ -655,12 +654,11 @@ DEV void shift_solve(const DenseCycle& d, int c, int i, c128* A, Sh& sh) {
     A[r + (long)me * lda] = cv[r];
     A[r + (long)(me + 1) * lda] = s[r];
   }
-  c128* tau = A + (long)lda * (me + 2);
-  c128* y = tau + (me + 1);
+  c128* y = A + (long)lda * (me + 2);
   c128* rinv = y + (me + 1);
   if (threadIdx.x == 0) sh.ibc[0] = 0;
   __syncthreads();
-  hess_qr(A, lda, rows, me, me + 2, tau, sh, d.kfull);
+  hess_qr(A, lda, rows, me, me + 2, sh, d.kfull);
   shift_finish(d, c, i, A, lda, beta, y, rinv, sh);
 }
 
