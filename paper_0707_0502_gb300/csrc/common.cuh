@@ -229,6 +229,13 @@ struct MvShape {
                       // g >= 2: the same within groups of g columns (pairs for the pair form)
 };
 
+// A 256-row tile of a CSR batch with all that its blocks need of their problem
+struct alignas(16) CsrTile {
+  long rp, nz;           // the problem's row pointers, and its columns and values, from here on
+  int problem, nrow;     // its number and its rows
+  int row0, pad;         // the tile's first row
+};
+
 struct gdr_op {
   gdr_ctx* ctx = nullptr;
   OpKind kind = OP_CSR;
@@ -245,7 +252,7 @@ struct gdr_op {
   long* rp_off = nullptr;
   long* nz_off = nullptr;
   int* nrow = nullptr;
-  int2* tiles = nullptr;  // every 256-row tile of every problem: {problem, tile}
+  CsrTile* tiles = nullptr;  // every 256-row tile of every problem
   long ntiles = 0;
   std::vector<long> nrow_host;
   // Wilson: links stored structure-of-arrays [mu][e][V], e = a*3 + b

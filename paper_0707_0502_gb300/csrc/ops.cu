@@ -90,31 +90,28 @@ __global__ void csr_kernel(long n, const int* __restrict__ rowptr, const int* __
 }
 
 // CSR batch: column c uses problem c / cpp (its own rows, local column indices).  The grid
-// holds the 256-row tiles the problems have (tiles: problem and tile), not the largest
-// problem's for all: of 64 problems with sides 32 to 256 two thirds of those were empty
-// (36.3 -> 35.0 us; requesting a row's entries together or staging them in shared memory
-// costs more occupancy than it hides: 37.6 and 46.7 us).  y: columns per problem; col_inner:
-// they are the fastest blocks instead.
+// holds the 256-row tiles the problems have, not the largest problem's for all: of 64 problems
+// with sides 32 to 256 two thirds of those were empty.  A tile's record holds its problem's
+// offsets, so that it takes the place of their loads in the chain a row waits for (record ->
+// row pointer -> column -> x) instead of lengthening it.  (Requesting a row's entries together
+// or staging them in shared memory costs more occupancy than it hides.)  y: columns per problem;
+// col_inner: they are the fastest blocks instead.
 template <typename R, typename VT, int TPR>
-__global__ void csr_batch_kernel(const long* __restrict__ rp_off, const long* __restrict__ nz_off,
-                                 const int* __restrict__ nrow, const int2* __restrict__ tiles,
+__global__ void csr_batch_kernel(const CsrTile* __restrict__ tiles, int sub_log2,
                                  const int* __restrict__ rowptr, const int* __restrict__ col,
                                  const VT* __restrict__ vals, const c128* __restrict__ sigma,
                                  const cx<R>* __restrict__ X, long ldx, cx<R>* __restrict__ Y, long ldy,
                                  const cx<R>* __restrict__ B, long ldb, const int* __restrict__ run, int run_stride,
                                  int cpp, const double* __restrict__ xs, int xs_stride, int ncol, int col_inner) {
-  const int sub = 256 / (blockDim.x / TPR);  // blocks of one 256-row tile
   const int t = col_inner ? blockIdx.x / cpp : blockIdx.x, k = col_inner ? blockIdx.x % cpp : blockIdx.y;
-  const int2 where = tiles[t / sub];  // problem, its tile
-  const int p = where.x, c = p * cpp + k;
-  if (c >= ncol) return;  // fewer columns than problems
-  const long tile = (long)where.y * sub + t % sub;
-  const long r = tile * (blockDim.x / TPR) + threadIdx.x / TPR;
-  if (r >= nrow[p]) return;
+  const CsrTile d = tiles[t >> sub_log2];  // 2^sub_log2 blocks to a tile
+  const int p = d.problem, c = p * cpp + k;
+  const int r = d.row0 + (t & ((1 << sub_log2) - 1)) * (int)(blockDim.x / TPR) + (int)(threadIdx.x / TPR);
+  if (c >= ncol || r >= d.nrow) return;  // fewer columns than problems; the last tile
   if (run && !run[(long)c * run_stride]) return;
-  const int* rp = rowptr + rp_off[p];
-  const int* cl = col + nz_off[p];
-  const VT* vl = vals + nz_off[p];
+  const int* rp = rowptr + d.rp;
+  const int* cl = col + d.nz;
+  const VT* vl = vals + d.nz;
   const cx<R>* x = X + c * ldx;
   cx<R> acc = {0, 0};
   const int p0 = rp[r], p1 = rp[r + 1];
@@ -505,10 +502,11 @@ static void csr_launch(gdr_ctx* ctx, const gdr_op* A, const VT* vals, const MvSh
         A->n, A->rowptr, A->col, vals, sigma, X, ldx, Y, ldy, B, ldb, run, run_stride, cpp, xs, xs_stride, ncol,
         s.col_inner);
   } else {
-    const long tiles = A->ntiles * (256 / rows);
-    csr_batch_kernel<R, VT, TPR><<<tile_grid(tiles, cpp, s.col_inner), s.threads, 0, ctx->stream>>>(
-        A->rp_off, A->nz_off, A->nrow, A->tiles, A->rowptr, A->col, vals, sigma, X, ldx, Y, ldy, B, ldb,
-        run, run_stride, cpp, xs, xs_stride, ncol, s.col_inner);
+    int sub_log2 = 0;  // 128 or 256 threads, 1 to 8 of them per row
+    while ((rows << sub_log2) < 256) ++sub_log2;
+    csr_batch_kernel<R, VT, TPR><<<tile_grid(A->ntiles << sub_log2, cpp, s.col_inner), s.threads, 0, ctx->stream>>>(
+        A->tiles, sub_log2, A->rowptr, A->col, vals, sigma, X, ldx, Y, ldy, B, ldb, run, run_stride, cpp, xs,
+        xs_stride, ncol, s.col_inner);
   }
   GDR_LAUNCHED(ctx);
 }
@@ -807,13 +805,13 @@ void op_build_csr_batch(gdr_ctx* ctx, gdr_op* op, const long* n, const long* nnz
                         const double* vals) {
   std::vector<long> rp(op->nprob), nz(op->nprob);
   std::vector<int> nr(op->nprob);
-  std::vector<int2> tiles;
+  std::vector<CsrTile> tiles;
   long rtot = 0, ztot = 0, nmax = 0;
   for (int p = 0; p < op->nprob; ++p) {
     rp[p] = rtot;
     nz[p] = ztot;
     nr[p] = (int)n[p];
-    for (long t = 0; t < (n[p] + 255) / 256; ++t) tiles.push_back(make_int2(p, (int)t));
+    for (long r0 = 0; r0 < n[p]; r0 += 256) tiles.push_back({rtot, ztot, p, (int)n[p], (int)r0, 0});
     rtot += n[p] + 1;
     ztot += nnz[p];
     nmax = std::max(nmax, n[p]);
@@ -828,9 +826,9 @@ void op_build_csr_batch(gdr_ctx* ctx, gdr_op* op, const long* n, const long* nnz
   GDR_CUDA(cudaMalloc(&op->rp_off, op->nprob * sizeof(long)));
   GDR_CUDA(cudaMalloc(&op->nz_off, op->nprob * sizeof(long)));
   GDR_CUDA(cudaMalloc(&op->nrow, op->nprob * sizeof(int)));
-  GDR_CUDA(cudaMalloc(&op->tiles, tiles.size() * sizeof(int2)));
+  GDR_CUDA(cudaMalloc(&op->tiles, tiles.size() * sizeof(CsrTile)));
   op->ntiles = (long)tiles.size();
-  GDR_CUDA(cudaMemcpyAsync(op->tiles, tiles.data(), tiles.size() * sizeof(int2), cudaMemcpyHostToDevice, ctx->stream));
+  GDR_CUDA(cudaMemcpyAsync(op->tiles, tiles.data(), tiles.size() * sizeof(CsrTile), cudaMemcpyHostToDevice, ctx->stream));
   GDR_CUDA(cudaMemcpyAsync(op->rowptr, rowptr, rtot * sizeof(int), cudaMemcpyDeviceToDevice, ctx->stream));
   if (ztot > 0) {
     GDR_CUDA(cudaMemcpyAsync(op->col, col, ztot * sizeof(int), cudaMemcpyDeviceToDevice, ctx->stream));
