@@ -421,6 +421,8 @@ gdr_status gdr_dense_restart(gdr_ctx *ctx, gdr_prec prec, int m, int k, const do
  * MIXED with 0 < nout, nv >= 54 and 26 <= nout + nx <= 64 (from 16 on with more than 60 vectors)
  * runs on the tensor cores (both factors split into two TF32 parts, FP32 accumulation: FP32
  * arithmetic's accuracy), below that on the CUDA cores in FP32; the call has no switch.
+ * There an infinite entry may give NaN where FP32 gives an infinity, and an entry below
+ * about 1e-34 in magnitude keeps TF32's 11 bits (its low part is subnormal).
  * A tensor-core wait that gave up is reported by the next call that synchronises
  * (GDR_ETIMEOUT, V and X then unspecified). */
 gdr_status gdr_basis_update(gdr_ctx *ctx, gdr_prec prec, long n, int nv, void *V, const double *C, int nout,
@@ -450,8 +452,10 @@ gdr_status gdr_basis_dot(gdr_ctx *ctx, gdr_prec prec, long n, int nv, const void
  * on the tensor cores with V and T split into two TF32 parts each (three
  * products, FP32 accumulation: the accuracy of FP32 arithmetic), unless flags
  * has GDR_FLAG_NO_TENSOR_CORES; otherwise the CUDA cores form it in FP32
- * (complex64) or FP64.  GDR_ETIMEOUT if a tensor-core wait gave up (R then
- * unspecified). */
+ * (complex64) or FP64.  On the tensor cores special values are as in
+ * gdr_basis_update, and the addition to R (of 16-byte aligned columns of even
+ * length and stride a reduction in L2) flushes subnormal values to zero.
+ * GDR_ETIMEOUT if a tensor-core wait gave up (R then unspecified). */
 gdr_status gdr_basis_residual_update(gdr_ctx *ctx, gdr_prec prec, long n, int nv, const void *V, int ncol,
                                      const double *T, void *R, long ldr, unsigned flags);
 

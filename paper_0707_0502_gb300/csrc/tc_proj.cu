@@ -941,12 +941,13 @@ bool tc_restart(gdr_ctx* ctx, long n, int ncol, c64* V, long ldv, long vcs, int 
   const int nn = nout + nx;
   tc_combine_sizes(a, nv);
   // The hand-overs per K atom cost the same however few outputs there are, the CUDA-core form's
-  // products grow with both, and its row tile of many vectors leaves fewer blocks on an SM; the
-  // vectors' length hardly moves the crossover.  us, CUDA cores -> here, at n = 3,072 / 49,152 /
-  // 786,432 (before whole tiles left by tensor stores, which only helps this side):
-  //   41 vectors, 20 outputs  10.8 -> 10.9 / 23.0 -> 25.1 / 233 -> 242;  26 outputs 1.06 / 1.07 / 1.13x
-  //   51 vectors, 20 outputs  0.86 / 0.93 / 0.99x;                       26 outputs 1.04 / 1.08 / 1.18x
-  //   61 vectors, 10 outputs  0.99 / 0.76 / 0.87x;                       15 outputs 1.09 / 1.09 / 1.17x
+  // products grow with both, and its row tile of many vectors leaves fewer blocks on an SM.  us,
+  // CUDA cores -> here, at n = 3,072 / 49,152 / 786,432:
+  //   54 vectors, 12 outputs   8.2 -> 10.3 / 19.5 -> 22.5 / 201 -> 215;  16  10.3 / 23.6 -> 22.9 / 248 -> 217
+  //               20 outputs  11.1 -> 12.2 / 28.7 -> 26.6 / 301 -> 260;  26  14.3 -> 12.3 / 37.9 -> 26.7 / 396 -> 261
+  //   61 vectors, 12 outputs  10.3 -> 10.3 / 20.7 -> 23.3 / 223 -> 220;  16  11.3 -> 10.3 / 28.9 -> 23.7 / 306 -> 220
+  //   81 vectors, 12 outputs  10.3 -> 12.3 / 29.5 -> 30.7 / 341 -> 313;  16  12.3 / 35.1 -> 30.7 / 406 -> 313
+  // 16 is the line above 60 vectors; up to 60 the line of 26 keeps to what wins at every length.
   // And the error: each MMA truncates where an FP32 FMA rounds, so this form's is about 1.4e-7 of
   // the result (rms) at any basis size, the CUDA cores' grows with the vectors: 1.04e-7 at 26, 1.25 at
   // 41, 1.38 at 51, 1.41 at 54 (here 1.36), 1.49 at 61 (1.41), 1.69 at 81 (1.41).
