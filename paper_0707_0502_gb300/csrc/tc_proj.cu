@@ -942,7 +942,7 @@ bool tc_restart(gdr_ctx* ctx, long n, int ncol, c64* V, long ldv, long vcs, int 
   tc_combine_sizes(a, nv);
   // The hand-overs per K atom cost the same however few outputs there are, the CUDA-core form's
   // products grow with both, and its row tile of many vectors leaves fewer blocks on an SM.  us,
-  // CUDA cores -> here, at n = 3,072 / 49,152 / 786,432:
+  // CUDA cores -> here (one figure: both), at n = 3,072 / 49,152 / 786,432:
   //   54 vectors, 12 outputs   8.2 -> 10.3 / 19.5 -> 22.5 / 201 -> 215;  16  10.3 / 23.6 -> 22.9 / 248 -> 217
   //               20 outputs  11.1 -> 12.2 / 28.7 -> 26.6 / 301 -> 260;  26  14.3 -> 12.3 / 37.9 -> 26.7 / 396 -> 261
   //   61 vectors, 12 outputs  10.3 -> 10.3 / 20.7 -> 23.3 / 223 -> 220;  16  11.3 -> 10.3 / 28.9 -> 23.7 / 306 -> 220
