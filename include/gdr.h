@@ -435,7 +435,7 @@ gdr_status gdr_basis_update(gdr_ctx *ctx, gdr_prec prec, long n, int nv, void *V
  * column stride ldr >= n; C: c128 nv x ncol (all device).  nv <= GDR_MAX_M + 1.
  * The complex64 form with ncol >= 8 runs on the tensor cores (TF32 inputs,
  * FP32 accumulation: each dot to about 1e-3 of ||v_i|| ||r_c||) when R and V
- * start on 16-byte boundaries, n and ldr are even and nv <= 128, unless flags has
+ * start on 16-byte boundaries, n < 2^30 and ldr are even and nv <= 128, unless flags has
  * GDR_FLAG_NO_TENSOR_CORES; otherwise the CUDA cores form it (FP32 products,
  * FP64 sums).  GDR_ETIMEOUT if a tensor-core wait gave up (C unspecified). */
 gdr_status gdr_basis_dot(gdr_ctx *ctx, gdr_prec prec, long n, int nv, const void *V, int ncol, const void *R,

@@ -846,6 +846,7 @@ int tc_proj_splits(gdr_ctx* ctx, long n, int ncol) {
 bool tc_proj_dot(gdr_ctx* ctx, long n, const c64* V, long ldv, int nv, const c64* R, long ldr, int ncol, c128* part,
                  int* err, int& nsplit, double prof_bytes) {
   if (nv < 1 || nv > TC_M || ncol < 1 || !ctx->tc_ok) return false;
+  if (n >= (1L << 30)) return false;  // TMA coordinates, in floats, are 32-bit
   const int ctiles = (ncol + 127) / 128;
   const int per = (ncol + ctiles - 1) / ctiles;
   const int nt = std::max(16, (per + 15) / 16 * 16);
