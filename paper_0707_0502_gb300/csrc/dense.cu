@@ -229,7 +229,7 @@ DEV void warp_givens_qr(c128* A, int lda, int rows, int j0, int cols, int ntot) 
 // (its own gives the norm), each by L lanes (4, 8 or 16, as many as keep all columns in a
 // pass), then, with v = x scal known, A[:, c] -= x (scal f_c), f_c = conj(tau) (A[j, c] +
 // conj(scal) d_c).  The scalars are formed by every thread for itself, two barriers a column.
-// A 41 x 40 system with six shifts: 1,110 -> 400 us, with dense_sh_cluster_kernel below.
+// A 41 x 40 system with six shifts: 1,110 -> 405 us, with dense_sh_cluster_kernel below.
 //
 // Every update forms its product first (A -= x h with one rounding of A): an entry passes through
 // up to 96 of them, and as FMA chains, two roundings each, they cost y and s 10 to 25% in error.
@@ -671,7 +671,7 @@ DEV void cluster_sync() {
 // a cluster of ns CTAs, the base solve in the first; the others factor their own shifted
 // matrices meanwhile, meet it at the cluster barrier, then take its s through the kept
 // reflectors.  As two launches the shifts' factorisations wait for the base solve (m = 40, six
-// shifts: 500 us, 351 in the cluster; 400 since the updates form their products first).
+// shifts: 500 us, 351 in the cluster; 405 since the updates form their products first).
 __global__ void __launch_bounds__(DT) dense_sh_cluster_kernel(DenseCycle d) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ Sh sh;
